@@ -19,9 +19,7 @@ fold_kernel(const float2 *__restrict__ ab, int I, int64_t ld, int J,
             int *__restrict__ status) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ fold_smem sm;
-    unsigned char *tab;
-    best_slots bs;
-    fold_smem_views(smem_raw, tab, bs);
+    unsigned char *tab = smem_raw + FT_RING_BYTES;
     const int t = threadIdx.x;
     const int jc = blockIdx.x / n_groups;
     const int grp = n_groups - 1 - (int)(blockIdx.x % n_groups);
@@ -40,11 +38,16 @@ fold_kernel(const float2 *__restrict__ ab, int I, int64_t ld, int J,
         sm.it.mask_k0 = k0;
         sm.it.gmax = FT_G;
     }
-    if (t < FT_G) fold_slot_meta(sm, t, k0 + t < K, k0 + t < K ? periods[k0 + t] : 0.0, I, c, p, q);
+    if (t < FT_G) {
+        // windows below what earlier chunks of the period found cannot be its maximum
+        const bool present = k0 + t < K;
+        fold_slot_meta(sm, t, present, present ? periods[k0 + t] : 0.0, I, c, p, q,
+                       present && accumulate ? (uint32_t)(__ldcg(&keys[k0 + t]) >> 32) : 0u);
+    }
     block_sync();
     ring rg;
     constexpr int R = KAHAN ? FT_R / 2 : FT_R;
-    fold_group<KAHAN, R>(sm, smem_raw, tab, bs, rg);
+    fold_group<KAHAN, R>(sm, smem_raw, tab, rg);
     block_sync();
     if (sm.abort) {
         drain_copies(sm, rg);
@@ -62,8 +65,7 @@ fold_kernel(const float2 *__restrict__ ab, int I, int64_t ld, int J,
 }  // namespace
 
 size_t fold_smem_bytes() {
-    return (size_t)FT_RING_BYTES + (size_t)FT_TAB_BYTES +
-           (size_t)FT_G * FT_THREADS * (sizeof(float) + sizeof(uint32_t));
+    return (size_t)FT_RING_BYTES + (size_t)FT_TAB_BYTES;
 }
 cudaError_t fold_configure() {
     const int bytes = (int)fold_smem_bytes();

@@ -116,12 +116,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// Candidate test of the epilogue: the exact comparison of a window's 2 LR = x^2 / y with the
-// running best b is x * __fdividef(x, y) > b, whose left side has a relative error below
-// 2^-21. With h = b (1 - 2^-14) and q = h y (each rounded once), fma(x, x, -q) > 0 (the exact
-// x^2 - q, rounded) holds whenever the exact comparison does (for b <= 0 trivially, for b > 0
-// by the margin), so a tile whose largest fma(x, x, -q) is not positive has no new maximum;
-// otherwise the exact comparison runs over the tile's windows in order, and decides as before.
+// Candidate test of the epilogue: a window enters the period's maximum when its
+// 2 LR = x * __fdividef(x, y), whose relative error is below 2^-21, is at least the largest so
+// far, b. With h = b (1 - 2^-14) and q = h y (each rounded once), fma(x, x, -q) > 0 (the exact
+// x^2 - q, rounded) holds for every window with 2 LR >= b > 0, by the margin, so a tile whose
+// largest fma(x, x, -q) is not positive holds none; otherwise the exact values decide.
 constexpr float kCandidate = 1.0f - 1.0f / 16384.0f;
 
 // ---------------------------------------------------------------------------------------------
@@ -143,6 +142,7 @@ struct fold_smem {
     uint64_t full[FT_NSTAGE];        // strip landed: the producer's arrival + the copy's bytes
     uint64_t empty[FT_NSTAGE];       // strip read: one arrival per consumer thread
     unsigned long long best[FT_G];   // best key of each slot of the group
+    __align__(16) int factor[FT_G];  // and its candidate test's factor (float bits)
     double P[FT_G], Ps[FT_G];        // period (days) and period in t0 steps
     int nph[FT_G], E[FT_G];          // phases, and an upper bound on the epochs with o_e < I
     int bad, tight;                  // table votes: spread too wide for the main / sliced path
@@ -277,50 +277,60 @@ __device__ __forceinline__ void issue_copy(fold_smem &sm, uint32_t ring0, const 
     bulk_load_s(ring0 + rg.stage * rg.bytes, src, bytes, &sm.full[rg.stage]);
 }
 
-// A consumer thread's running maximum of each period of the sub-group, in shared memory: slot
-// gg of thread c at [gg * FT_THREADS + c], the largest 2 LR so far and the flat index of its
-// window. They are read once per tile and written only when a maximum changes, so they take
-// no registers in the hot loop.
-struct best_slots {
-    float *lr2;
-    uint32_t *at;
-};
+// The running maximum of a period is the block's: the slot's best key in shared memory. Every
+// warp tests its tile's windows against it (load_factors, kCandidate) and works out exact values only
+// when one of them may reach it. A maximum kept per thread is beaten again and again (the k-th
+// tile of a thread beats its earlier ones with probability 1/k, and one lane in 32 is enough to
+// send the warp through the exact values); the block's is beaten a few times per period.
 
+// The factors h of the candidate test live beside the keys, as ordered integers: h is -1 (every
+// window with data is a candidate) while a slot has no maximum above zero, so that the first of
+// equal zeros is found, and stays there if the maximum is not finite.
+__device__ __forceinline__ float candidate_factor(uint32_t lr_bits) {
+    const float b = 2.0f * __uint_as_float(lr_bits);
+    return b > 0.0f && b < INFINITY ? b * kCandidate : -1.0f;
+}
 template <int GS>
-__device__ __forceinline__ void init_best(best_slots bs) {
+__device__ __forceinline__ void load_factors(const fold_smem &sm, int g0, float (&h)[GS]) {
+    const uint32_t a = smem_u32(&sm.factor[g0]);
+    if constexpr (GS >= 4) {
 #pragma unroll
-    for (int gg = 0; gg < GS; ++gg) {
-        bs.lr2[gg * FT_THREADS + threadIdx.x] = -1.0f;
-        bs.at[gg * FT_THREADS + threadIdx.x] = 0u;
+        for (int g = 0; g < GS; g += 4)
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(h[g]), "=f"(h[g + 1]), "=f"(h[g + 2]), "=f"(h[g + 3])
+                         : "r"(a + 4u * g));
+    } else {
+#pragma unroll
+        for (int g = 0; g < GS; ++g)
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(h[g]) : "r"(a + 4u * g));
     }
 }
 
-// Per-thread best of each period (the largest 2 LR, first in (j, i) order on ties) -> the
-// slot's best key in shared memory.
-template <int GS>
-__device__ __forceinline__ void publish_best(fold_smem &sm, int g0, best_slots bs) {
-    const int c = threadIdx.x;
-#pragma unroll
-    for (int gg = 0; gg < GS; ++gg) {
-        const float b = bs.lr2[gg * FT_THREADS + c];
-        unsigned long long key = b >= 0.0f ? make_key(0.5f * b, bs.at[gg * FT_THREADS + c]) : 0ull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long u = __shfl_xor_sync(0xFFFFFFFFu, key, o);
-            key = u > key ? u : key;
+// Offer slot g the best window of each lane of a warp (called by whole warps): 2 LR = lr2 at
+// flat index at; a lane without one passes lr2 < 0. The larger LR stays, on equal LR the smaller
+// flat index (make_key).
+__device__ __forceinline__ void offer_best(fold_smem &sm, int g, float lr2, uint32_t at) {
+    const uint32_t v = lr2 >= 0.0f ? __float_as_uint(0.5f * lr2) + 1u : 0u;  // 0: none
+    const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, v);
+    if (top == 0u) return;
+    if (v == top) {  // one lane, or a few equal ones: the key decides
+        const unsigned long long key =
+            ((unsigned long long)(top - 1u) << 32) | (unsigned long long)(0xFFFFFFFFu - at);
+        if (key > *(volatile unsigned long long *)&sm.best[g]) {
+            atomicMax(&sm.best[g], key);
+            atomicMax(&sm.factor[g], __float_as_int(candidate_factor(top - 1u)));
         }
-        if ((threadIdx.x & 31) == 0 && key) atomicMax(&sm.best[g0 + gg], key);
     }
 }
 
-// Exact running maximum over one window sum (x, y) = (sum A, sum B) at flat index at:
-// 2 LR = x * (x / y); a null sum gives NaN, never a maximum; the first of equal values stays.
-__device__ __forceinline__ void take_max(float x, float y, uint32_t at, best_slots bs, int gg) {
-    const int k = gg * FT_THREADS + threadIdx.x;
-    const float lr2 = x * __fdividef(x, y);
-    if (lr2 > bs.lr2[k]) {
-        bs.lr2[k] = lr2;
-        bs.at[k] = at;
+// The better of a lane's best window (lr2, at) and the window sum (x, y) at index here, which
+// comes later in flat order: 2 LR = x * (x / y); a null sum gives NaN, never a maximum.
+__device__ __forceinline__ void take_max(float x, float y, uint32_t here, float &lr2,
+                                         uint32_t &at) {
+    const float v = x * __fdividef(x, y);
+    if (v > lr2) {
+        lr2 = v;
+        at = here;
     }
 }
 
@@ -447,7 +457,7 @@ __device__ __forceinline__ bool consume_epochs(fold_smem &sm, const fold_table &
 template <int GS, int R, int W, bool KAHAN, bool SHORT>
 __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb, int g0, int j,
                                              int i0, int nE, unsigned use, bool all_used,
-                                             int nmin, uint32_t mine, best_slots bs, ring &rg) {
+                                             int nmin, uint32_t mine, ring &rg) {
     constexpr int T = FT_THREADS * R;
     const int c = threadIdx.x;
     uint64_t acc[GS][R];
@@ -523,39 +533,41 @@ __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb
                      : consume_epochs<GS, R, W, KAHAN, false>(sm, tb, nE, use, mine, acc, cmp, rg);
         if (!ok) return false;
     }
-    // 2 LR = SA^2 / SB per (period, phase); the running maximum keeps the first (smallest j,
-    // then smallest i) of equal values. Whole tiles (nmin: the phases every used period has)
-    // first run the candidate test over all their windows.
+    // 2 LR = SA^2 / SB per (period, phase). Whole tiles (nmin: the phases every used period
+    // has) first run the candidate test over all their windows.
     float m = i0 + T > nmin ? 1.0f : -1.0f;  // a ragged tile takes the exact comparisons
+    float h[GS];
+    load_factors<GS>(sm, g0, h);
 #pragma unroll
     for (int gg = 0; gg < GS; ++gg) {
         if (!all_used && !((use >> gg) & 1u)) continue;
-        const float h = bs.lr2[gg * FT_THREADS + c] * kCandidate;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             uint64_t v = acc[gg][r];
             if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
             float x, y;
             split_pair(v, x, y);
-            m = fmaxf(m, fmaf(x, x, -(h * y)));
+            m = fmaxf(m, fmaf(x, x, -(h[gg] * y)));
         }
     }
-    if (m > 0.0f) {
-        const uint32_t jI = (uint32_t)j * (uint32_t)sm.it.I;
+    if (__any_sync(0xFFFFFFFFu, m > 0.0f)) {
+        const uint32_t at0 = (uint32_t)j * (uint32_t)sm.it.I + (uint32_t)(i0 + c);
 #pragma unroll
         for (int gg = 0; gg < GS; ++gg) {
             if (!((use >> gg) & 1u)) continue;
             const int nph = sm.nph[g0 + gg];
+            float lr2 = -1.0f;
+            uint32_t at = 0u;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const int i = i0 + c + r * FT_THREADS;
                 uint64_t v = acc[gg][r];
                 if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
                 float x, y;
                 split_pair(v, x, y);
-                if (i < nph)
-                    take_max(x, y, jI + (uint32_t)i, bs, gg);
+                if (i0 + c + r * FT_THREADS < nph)
+                    take_max(x, y, at0 + (uint32_t)(r * FT_THREADS), lr2, at);
             }
+            offer_best(sm, g0 + gg, lr2, at);
         }
     }
     return true;
@@ -567,25 +579,24 @@ template <int GS, int R, int W, bool KAHAN, int RL>
 __device__ __forceinline__ bool consume_tile_rows(int rows, fold_smem &sm, const fold_table &tb,
                                                   int g0, int j, int i0, int nE, unsigned use,
                                                   bool all_used, int nmin, uint32_t mine,
-                                                  best_slots bs, ring &rg) {
+                                                  ring &rg) {
     if constexpr (RL > 1 && GS >= 4) {
         if (rows < RL)
             return consume_tile_rows<GS, R, W, KAHAN, RL - 1>(rows, sm, tb, g0, j, i0, nE, use,
-                                                              all_used, nmin, mine, bs, rg);
+                                                              all_used, nmin, mine, rg);
     }
     return nE <= 3 ? consume_tile<GS, RL, W, KAHAN, true>(sm, tb, g0, j, i0, nE, use, all_used,
-                                                          nmin, mine, bs, rg)
+                                                          nmin, mine, rg)
                    : consume_tile<GS, RL, W, KAHAN, false>(sm, tb, g0, j, i0, nE, use, all_used,
-                                                           nmin, mine, bs, rg);
+                                                           nmin, mine, rg);
 }
 
 template <int GS, int R, int W, bool KAHAN>
-__device__ void consume_main(fold_smem &sm, uint32_t ring0, best_slots bs, const fold_table &tb,
+__device__ void consume_main(fold_smem &sm, uint32_t ring0, const fold_table &tb,
                              int g0, int nph_sub, ring &rg) {
     constexpr int T = FT_THREADS * R;
     const int c = threadIdx.x;
     const uint32_t mine = ring0 + (uint32_t)c * (uint32_t)sizeof(float2);
-    init_best<GS>(bs);
     for (int j = sm.it.jlo; j < sm.it.jhi; ++j) {
         const unsigned use = period_use<GS>(sm, g0, j);
         if (!use) continue;
@@ -601,11 +612,10 @@ __device__ void consume_main(fold_smem &sm, uint32_t ring0, best_slots bs, const
             // so every thread still meets the caller's next one)
             const bool ok = consume_tile_rows<GS, R, W, KAHAN, R>(
                 tile_rows<GS, R>(nph_sub - i0), sm, tb, g0, j, i0, nE, use, all_used, nmin, mine,
-                bs, rg);
+                rg);
             if (!ok) return;
         }
     }
-    publish_best<GS>(sm, g0, bs);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -655,7 +665,7 @@ __device__ void produce_sliced(fold_smem &sm, uint32_t ring0, const fold_table &
 }
 
 template <int GS, int R, int W, bool KAHAN>
-__device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part, best_slots bs,
+__device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part,
                                const fold_table &tb, int g0, int Tp, ring &rg) {
     constexpr int T = FT_THREADS * R;
     const int H = T / Tp;
@@ -668,7 +678,6 @@ __device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part, be
         slice[r] = L / Tp;
         phase[r] = L - slice[r] * Tp;
     }
-    init_best<GS>(bs);
     for (int j = sm.it.jlo; j < sm.it.jhi; ++j) {
         const unsigned use = period_use<GS>(sm, g0, j);
         if (!use) continue;
@@ -727,18 +736,20 @@ __device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part, be
             }
             block_sync();
             const int nph = sm.nph[g0 + gg];
-            for (int phi = c; phi < Tp; phi += FT_THREADS) {
+            float lr2 = -1.0f;
+            uint32_t at = 0u;
+            for (int phi = c; phi < min(Tp, nph); phi += FT_THREADS) {
                 uint64_t v = part[phi];
                 for (int h = 1; h < H; ++h) add_pair(v, part[h * Tp + phi]);
                 float x, y;
                 split_pair(v, x, y);
-                if (phi < nph && y > 0.0f)
-                    take_max(x, y, (uint32_t)j * (uint32_t)I + (uint32_t)phi, bs, gg);
+                take_max(x, y, (uint32_t)j * (uint32_t)I + (uint32_t)phi, lr2, at);
             }
+            if (__any_sync(0xFFFFFFFFu, lr2 > __int_as_float(*(volatile int *)&sm.factor[g0 + gg])))
+                offer_best(sm, g0 + gg, lr2, at);
             block_sync();
         }
     }
-    publish_best<GS>(sm, g0, bs);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -801,7 +812,7 @@ __device__ void produce_packed(fold_smem &sm, uint32_t ring0, const fold_table &
 }
 
 template <int GS, int R, int W, bool KAHAN>
-__device__ void consume_packed(fold_smem &sm, uint32_t ring0, best_slots bs, const fold_table &tb,
+__device__ void consume_packed(fold_smem &sm, uint32_t ring0, const fold_table &tb,
                                int g0, int Tp, int H, int seg, ring &rg) {
     const int c = threadIdx.x;
     const int nJ = sm.pack_n;
@@ -818,7 +829,6 @@ __device__ void consume_packed(fold_smem &sm, uint32_t ring0, best_slots bs, con
                                    (uint32_t)sizeof(float2)
                              : 0u;  // idle lane: reads row 0, never used
     }
-    init_best<GS>(bs);
     for (int t0 = 0; t0 < nJ; t0 += H) {
         const int nr = min(H, nJ - t0);
         uint64_t acc[GS][R];
@@ -864,25 +874,42 @@ __device__ void consume_packed(fold_smem &sm, uint32_t ring0, best_slots bs, con
             mbar_arrive(&sm.empty[rg.stage]);
             rg.next();
         }
-        // running maxima, in (duration, phase) order within the thread
+        // maxima, the lane's windows in (duration, phase) order
+        unsigned use[R];
+        float m = -1.0f;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            if (row[r] >= nr) continue;
-            const int k = t0 + row[r];
-            const uint32_t at = (uint32_t)sm.pack_j[k] * I + (uint32_t)ph[r];
-            const unsigned u = sm.pack_use[k];
+        for (int r = 0; r < R; ++r) use[r] = row[r] < nr ? sm.pack_use[t0 + row[r]] : 0u;
+        float h[GS];
+        load_factors<GS>(sm, g0, h);
 #pragma unroll
-            for (int gg = 0; gg < GS; ++gg) {
-                if (!((u >> gg) & 1u) || ph[r] >= sm.nph[g0 + gg]) continue;
+        for (int gg = 0; gg < GS; ++gg) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
                 uint64_t v = acc[gg][r];
                 if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
                 float x, y;
                 split_pair(v, x, y);
-                take_max(x, y, at, bs, gg);
+                if ((use[r] >> gg) & 1u) m = fmaxf(m, fmaf(x, x, -(h[gg] * y)));
             }
         }
+        if (!__any_sync(0xFFFFFFFFu, m > 0.0f)) continue;
+#pragma unroll
+        for (int gg = 0; gg < GS; ++gg) {
+            float lr2 = -1.0f;
+            uint32_t at = 0u;
+            const int nph = sm.nph[g0 + gg];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (!((use[r] >> gg) & 1u) || ph[r] >= nph) continue;
+                uint64_t v = acc[gg][r];
+                if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
+                float x, y;
+                split_pair(v, x, y);
+                take_max(x, y, (uint32_t)sm.pack_j[t0 + row[r]] * I + (uint32_t)ph[r], lr2, at);
+            }
+            offer_best(sm, g0 + gg, lr2, at);
+        }
     }
-    publish_best<GS>(sm, g0, bs);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -920,9 +947,11 @@ __device__ void fold_direct(fold_smem &sm, int g) {
 // ---------------------------------------------------------------------------------------------
 
 // Slot t of a group (thread t < FT_G): P, Ps = P/s in t0 steps, the number of phases and an
-// upper bound on the epochs with o_e < I.
+// upper bound on the epochs with o_e < I. floor_lr: the LR (float bits) below which a window is
+// of no interest to the caller (0: every window is).
 __device__ __forceinline__ void fold_slot_meta(fold_smem &sm, int t, bool present, double P,
-                                               int I, double c, int64_t p, int64_t q) {
+                                               int I, double c, int64_t p, int64_t q,
+                                               uint32_t floor_lr) {
     double Ps = 0.0;
     int nph = 0, E = 0;
     if (present) {
@@ -942,6 +971,7 @@ __device__ __forceinline__ void fold_slot_meta(fold_smem &sm, int t, bool presen
     sm.nph[t] = nph;
     sm.E[t] = E;
     sm.best[t] = 0ull;
+    sm.factor[t] = __float_as_int(candidate_factor(floor_lr));
 }
 
 // Build the epoch table of sub-group [g0, g0 + GS) (all threads), offsets W bytes wide. Sets
@@ -1004,7 +1034,7 @@ __device__ __forceinline__ void build_table_w(fold_smem &sm, unsigned char *raw,
 
 template <int GS, int R, int W, bool KAHAN>
 __device__ void fold_subgroup(fold_smem &sm, uint32_t ring0, const fold_table &tb, uint64_t *part,
-                              best_slots bs, bool sliced, int Tp, int g0, int nph_sub, int H,
+                              bool sliced, int Tp, int g0, int nph_sub, int H,
                               int seg, ring &rg) {
     const bool producer = threadIdx.x >= FT_THREADS;
     if (H > 0) {
@@ -1014,33 +1044,33 @@ __device__ void fold_subgroup(fold_smem &sm, uint32_t ring0, const fold_table &t
                 if ((threadIdx.x & 31) == 0) produce_packed(sm, ring0, tb, Tp, H, seg, rg);
                 __syncwarp();
             } else {
-                consume_packed<GS, R, W, KAHAN>(sm, ring0, bs, tb, g0, Tp, H, seg, rg);
+                consume_packed<GS, R, W, KAHAN>(sm, ring0, tb, g0, Tp, H, seg, rg);
             }
         }
     } else if (sliced) {
         if (producer)
             produce_sliced<GS, R>(sm, ring0, tb, g0, Tp, rg);
         else
-            consume_sliced<GS, R, W, KAHAN>(sm, ring0, part, bs, tb, g0, Tp, rg);
+            consume_sliced<GS, R, W, KAHAN>(sm, ring0, part, tb, g0, Tp, rg);
     } else if (producer) {
         // the main path has no block barrier: the producer's first lane runs it alone
         if ((threadIdx.x & 31) == 0) produce_main<GS, R>(sm, ring0, tb, g0, nph_sub, rg);
         __syncwarp();
     } else {
-        consume_main<GS, R, W, KAHAN>(sm, ring0, bs, tb, g0, nph_sub, rg);
+        consume_main<GS, R, W, KAHAN>(sm, ring0, tb, g0, nph_sub, rg);
     }
 }
 
 template <int GS, int R, bool KAHAN>
 __device__ __forceinline__ void fold_subgroup_w(fold_smem &sm, uint32_t ring0,
                                                 const fold_table &tb, uint64_t *part,
-                                                best_slots bs, bool sliced, int Tp, int g0,
+                                                bool sliced, int Tp, int g0,
                                                 int nph_sub, int H, int seg, ring &rg, int W) {
     if (W == 4)
-        fold_subgroup<GS, R, 4, KAHAN>(sm, ring0, tb, part, bs, sliced, Tp, g0, nph_sub, H, seg,
+        fold_subgroup<GS, R, 4, KAHAN>(sm, ring0, tb, part, sliced, Tp, g0, nph_sub, H, seg,
                                        rg);
     else
-        fold_subgroup<GS, R, 2, KAHAN>(sm, ring0, tb, part, bs, sliced, Tp, g0, nph_sub, H, seg,
+        fold_subgroup<GS, R, 2, KAHAN>(sm, ring0, tb, part, sliced, Tp, g0, nph_sub, H, seg,
                                        rg);
 }
 
@@ -1048,7 +1078,7 @@ __device__ __forceinline__ void fold_subgroup_w(fold_smem &sm, uint32_t ring0,
 // (8 -> 4 -> 2 -> 1 periods, as the table allows) in turn; slot g's best key ends in
 // sm.best[g]. A wait that gave up leaves sm.abort set.
 template <bool KAHAN, int R>
-__device__ __forceinline__ void fold_group(fold_smem &sm, unsigned char *raw, unsigned char *tab, best_slots bs,
+__device__ __forceinline__ void fold_group(fold_smem &sm, unsigned char *raw, unsigned char *tab,
                            ring &rg) {
     constexpr int T = FT_THREADS * R;
     for (int g0 = 0; g0 < FT_G;) {
@@ -1129,7 +1159,7 @@ __device__ __forceinline__ void fold_group(fold_smem &sm, unsigned char *raw, un
             const int Tq = (nph_sub + 1) & ~1;
             const int sq = Tq + 32 * ((sm.spread + 3 + 31) / 32);
             int Hq = min(T / Tq, nJ);
-            Hq = min(Hq, (int)(FT_RING_BYTES / (2u * (uint32_t)sq * (uint32_t)sizeof(float2))));
+            Hq = min(Hq, (int)(FT_PACK_BYTES / (2u * (uint32_t)sq * (uint32_t)sizeof(float2))));
             const int tiles = Hq > 0 ? (nJ + Hq - 1) / Hq : 0;
             if (Hq >= 2 && 2 * nJ * Tq >= tiles * T) {
                 H = Hq;
@@ -1143,16 +1173,16 @@ __device__ __forceinline__ void fold_group(fold_smem &sm, unsigned char *raw, un
         uint64_t *part = reinterpret_cast<uint64_t *>(raw + (ns - 1) * stage_bytes);
         const uint32_t ring0 = smem_u32(raw);
         if (GS == 8)
-            fold_subgroup_w<8, R, KAHAN>(sm, ring0, tb, part, bs, sliced, Tp, g0, nph_sub, H, seg,
+            fold_subgroup_w<8, R, KAHAN>(sm, ring0, tb, part, sliced, Tp, g0, nph_sub, H, seg,
                                          rg, W);
         else if (GS == 4)
-            fold_subgroup_w<4, R, KAHAN>(sm, ring0, tb, part, bs, sliced, Tp, g0, nph_sub, H, seg,
+            fold_subgroup_w<4, R, KAHAN>(sm, ring0, tb, part, sliced, Tp, g0, nph_sub, H, seg,
                                          rg, W);
         else if (GS == 2)
-            fold_subgroup_w<2, R, KAHAN>(sm, ring0, tb, part, bs, sliced, Tp, g0, nph_sub, H, seg,
+            fold_subgroup_w<2, R, KAHAN>(sm, ring0, tb, part, sliced, Tp, g0, nph_sub, H, seg,
                                          rg, W);
         else
-            fold_subgroup_w<1, R, KAHAN>(sm, ring0, tb, part, bs, sliced, Tp, g0, nph_sub, H, seg,
+            fold_subgroup_w<1, R, KAHAN>(sm, ring0, tb, part, sliced, Tp, g0, nph_sub, H, seg,
                                          rg, W);
         g0 += GS;
     }
@@ -1179,12 +1209,6 @@ __device__ void drain_copies(fold_smem &sm, const ring &rg) {
     for (int s = 0; s < FT_NSTAGE; ++s) mbar_wait(&sm.full[s], ((rg.par >> s) & 1u) ^ 1u);
 }
 
-// Dynamic shared memory: the strip ring, the epoch table, the consumers' running maxima.
-__device__ __forceinline__ void fold_smem_views(unsigned char *raw, unsigned char *&tab,
-                                                best_slots &bs) {
-    tab = raw + FT_RING_BYTES;
-    bs.lr2 = reinterpret_cast<float *>(tab + FT_TAB_BYTES);
-    bs.at = reinterpret_cast<uint32_t *>(bs.lr2 + FT_G * FT_THREADS);
-}
+// Dynamic shared memory: the strip ring, then the epoch table.
 
 }  // namespace

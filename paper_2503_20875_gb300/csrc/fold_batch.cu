@@ -27,9 +27,7 @@ batch_fold_kernel(const float2 *__restrict__ ab, const batch_curve *__restrict__
     __shared__ int s_item;
     // the queue length: n_items, or the count a device-side selection left (capped by n_items)
     if (n_items_dev) n_items = min(n_items, (int64_t)*n_items_dev);
-    unsigned char *tab;
-    best_slots bs;
-    fold_smem_views(smem_raw, tab, bs);
+    unsigned char *tab = smem_raw + FT_RING_BYTES;
     const int t = threadIdx.x;
     fold_init_barriers(sm);
     ring rg;
@@ -65,11 +63,12 @@ batch_fold_kernel(const float2 *__restrict__ ab, const batch_curve *__restrict__
         }
         if (t < FT_G) {
             const bool present = k0 + t < cv.n_periods;
+            // only windows that reach the curve's best so far matter: its key keeps the larger
             fold_slot_meta(sm, t, present, present ? batch_period(cv.pmin, cv.ratio, k0 + t) : 0.0,
-                           cv.I, c, p, q);
+                           cv.I, c, p, q, (uint32_t)(__ldcg(&curve_keys[cidx]) >> 32));
         }
         block_sync();
-        fold_group<KAHAN, R>(sm, smem_raw, tab, bs, rg);
+        fold_group<KAHAN, R>(sm, smem_raw, tab, rg);
         block_sync();
         if (sm.abort) {
             drain_copies(sm, rg);

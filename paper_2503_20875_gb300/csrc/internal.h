@@ -114,8 +114,9 @@ constexpr int LIN_SUB = 16;  // register blocks per partial sum of the linear ke
 #define FT_NSTAGE 8       // strips in flight per block at most (as many as the ring holds)
 #endif
 #ifndef FT_RING_BYTES
-#define FT_RING_BYTES (56 * 1024)  // strip ring: FT_RING_BYTES / strip bytes stages, <= FT_NSTAGE
+#define FT_RING_BYTES (70 * 1024)  // strip ring: FT_RING_BYTES / strip bytes stages, <= FT_NSTAGE
 #endif
+constexpr int FT_PACK_BYTES = 56 * 1024;  // rows of a duration-packed tile: two strips fit this
 #ifndef FT_MIN_BLOCKS
 #define FT_MIN_BLOCKS 2
 #endif
