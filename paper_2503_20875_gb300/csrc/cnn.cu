@@ -10,12 +10,14 @@
 // weight w+), Adam. All kernels are written here; nothing calls a library.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
 #include <random>
 #include <vector>
 
+#include "device.cuh"
 #include "internal.h"
 
 namespace {
@@ -31,13 +33,6 @@ constexpr int CONV_THREADS = (CONV_TT / CONV_RT) * (CNN_C / CONV_RC);  // 128
 constexpr size_t kCombSmemMax = 96 * 1024;  // maps up to 24,576 bins are staged in shared memory
 
 // ------------------------------------------------------------------------------- kernels
-
-// x0 = log1p(max(f, 0))
-__global__ void cnn_prep_kernel(const float *__restrict__ f, float *__restrict__ x, int64_t n) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        x[i] = log1pf(fmaxf(f[i], 0.0f));
-}
 
 // y[b][co][t] = act(bias[co] + sum_ci sum_k w[co][ci][k] x[b][ci][t + k - 4]), zero padding.
 // One block: all output channels (cout <= 32) of CONV_TT bins of one curve. Thread:
@@ -99,6 +94,337 @@ cnn_conv_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w
             yb[(int64_t)co * T + t0 + tt + r] = v;
         }
     }
+}
+
+// ------------------------------------------------------------------------- fused forward pass
+//
+// All four layers of NET_OUT bins of one curve per tile, on the tensor cores (tcgen05), without
+// the activations leaving the SM (training also stores them). Conv as GEMM: D[bin][co] +=
+// X[bin + k][ci] W[k][ci][co] for the 9 taps k: the activations sit in shared memory as rows
+// (bins) of 8-channel units of 16 bytes, every row 16 bytes after the one before it, so a tap is
+// a row offset of the operand's start address and nothing is gathered. M = 128 bins, N = 32
+// channels, K = 16 channels per instruction.
+//
+// Precision: the weights are BF16 values; an FP32 activation is the exact sum of three BF16
+// parts (its leading 8, middle 8 and last 8 bits), so three products with the same weight give
+// the FP32 product exactly. The tensor core's accumulator truncates, so a sum is kept in NET_GRP
+// accumulators (taps 0-1, 2-3, 4-5, 6-8; each takes its last and middle parts first), which are
+// added in FP32. Measured error of the probabilities against 64 bits: see cnn_forward.
+//
+// Halo: layer l's row r is bin t0 - 16 + 4 l + r. A tile computes NET_ROWS = 256 rows of the
+// first three layers in place (rows past the last valid one are never used): 256, 248, 240
+// valid rows, then NET_OUT = 232 logits. Rows outside [0, T) are zero (zero padding).
+//
+// Bound: the shared-memory reads of the activation operand (4 KB, 32 clocks per instruction,
+// against 16 of arithmetic): 270 instructions per tile at 16 durations. Two blocks per SM, so
+// that one's epilogue runs under the other's matrix instructions.
+constexpr int NET_ROWS = 256;              // rows computed per layer (two M = 128 blocks)
+constexpr int NET_XROWS = NET_ROWS + 8;    // rows held: 8 more for the last tap
+constexpr int NET_OUT = NET_ROWS - 24;     // logits per tile
+constexpr int NET_THREADS = 256;
+constexpr int NET_GRP = 4;                 // accumulators of a sum
+constexpr int NET_UNIT = NET_XROWS * 16;   // bytes of one 8-channel unit of all rows
+constexpr int NET_PART = 4 * NET_UNIT;     // bytes of one BF16 part (32 channels)
+constexpr int NET_ACT3_LD = 260;           // floats per channel row of the last activation
+constexpr int NET_TMEM_COLS = 2 * NET_GRP * CNN_C;  // 256
+static_assert(3 * NET_PART >= CNN_C * NET_ACT3_LD * 4 + 4 * NET_ROWS * 4, "activation reuse");
+
+__host__ __device__ constexpr int net_units(int cin) { return (cin + 15) / 16 * 2; }
+// bytes of the BF16 weights of a layer with `units` input units: [tap][unit][co][8 ci]
+__host__ __device__ constexpr int net_wbytes(int units) { return CNN_K * units * CNN_C * 16; }
+inline size_t net_smem(int cin) {
+    return (size_t)3 * NET_PART + net_wbytes(net_units(cin)) + 2 * net_wbytes(4) +
+           (CNN_C * CNN_K + 4 * CNN_C) * sizeof(float);
+}
+
+struct net_layers {
+    const __nv_bfloat16 *w[CNN_LAYERS];  // [co][ci][9], BF16
+    const float *bias[CNN_LAYERS];
+    float *act[CNN_LAYERS + 1];          // training: log1p(features), the activations, the logits
+};
+
+// Matrix descriptor of a K-major operand without swizzle: rows 16 bytes apart, 8-row groups 128
+// bytes apart, the second 8-element unit of K `unit_bytes` after the first.
+__device__ __forceinline__ uint64_t net_desc(uint32_t addr, uint32_t unit_bytes) {
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(unit_bytes >> 4) << 16) |
+           ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+
+// kind::f16: FP32 accumulator, BF16 operands, both K-major, M = 128, N = 32.
+constexpr uint32_t NET_IDESC =
+    (1u << 4) | (1u << 7) | (1u << 10) | ((CNN_C / 8) << 17) | ((128 / 16) << 24);
+
+__device__ __forceinline__ void net_mma(uint32_t d, uint64_t a, uint64_t b, bool add) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(NET_IDESC), "r"((uint32_t)add)
+        : "memory");
+}
+__device__ __forceinline__ void net_commit(uint64_t *bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+            smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void net_tmem_load(float (&v)[16], uint32_t taddr) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+          "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
+}
+// Wait for the warp's loads; the operands tie the uses of the loaded values to the wait.
+__device__ __forceinline__ void net_tmem_wait(float (&v)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]),
+                   "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]),
+                   "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
+                 :
+                 : "memory");
+}
+
+// Eight channels of one row as three BF16 parts (the leading, middle and last 8 bits of each
+// value: exact) into the 16-byte slot at `at` of every part.
+__device__ __forceinline__ void net_store_row(uint32_t at, const float *v) {
+    uint32_t p[3][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t part[3][2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float x = v[2 * k + e];
+            const uint32_t hi = __float_as_uint(x) & 0xFFFF0000u;
+            float r = x - __uint_as_float(hi);
+            if (!(fabsf(x) < INFINITY)) r = 0.0f;  // an infinity or NaN is its leading part
+            const uint32_t mid = __float_as_uint(r) & 0xFFFF0000u;
+            part[0][e] = hi;
+            part[1][e] = mid;
+            part[2][e] = __float_as_uint(r - __uint_as_float(mid));
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) p[q][k] = __byte_perm(part[q][0], part[q][1], 0x7632);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + q * NET_PART),
+                     "r"(p[q][0]), "r"(p[q][1]), "r"(p[q][2]), "r"(p[q][3])
+                     : "memory");
+}
+
+template <bool STORE>
+__global__ void __launch_bounds__(NET_THREADS, 2)
+cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__restrict__ prob,
+               int cin, int T, int n_tiles, int tiles_per_curve) {
+    extern __shared__ __align__(128) unsigned char net_raw[];
+    __shared__ uint64_t done[2];  // matrix instructions of row block 0 / 1 complete
+    __shared__ uint32_t s_tmem;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int units1 = net_units(cin);
+    const uint32_t x0 = smem_u32(net_raw);
+    unsigned char *wraw = net_raw + 3 * NET_PART;
+    const uint32_t w0 = x0 + 3 * NET_PART;
+    const int wsize1 = net_wbytes(units1);
+    float *w4 = reinterpret_cast<float *>(wraw + wsize1 + 2 * net_wbytes(4));  // [co][9]
+    float *bias = w4 + CNN_C * CNN_K;                                          // [4][32]
+    float *act3 = reinterpret_cast<float *>(net_raw);    // [32][NET_ACT3_LD], after layer 3
+    float *part = act3 + CNN_C * NET_ACT3_LD;            // [4][NET_ROWS]
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(&s_tmem)),
+                     "n"(NET_TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        mbar_init(&done[0], 1);
+        mbar_init(&done[1], 1);
+        fence_mbar_init();
+    }
+    // weights: [tap][unit][co][8 ci] (channels past the layer's own are zero)
+    for (int l = 0; l < 3; ++l) {
+        const int ci_n = l == 0 ? cin : CNN_C, units = l == 0 ? units1 : 4;
+        __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(
+            wraw + (l == 0 ? 0 : wsize1 + (l - 1) * net_wbytes(4)));
+        const int n = CNN_K * units * CNN_C * 8;
+        for (int i = tid; i < n; i += NET_THREADS) {
+            const int e = i & 7, co = (i >> 3) & 31, ku = i >> 8;
+            const int ci = (ku % units) * 8 + e, k = ku / units;
+            dst[i] = ci < ci_n ? net.w[l][(co * ci_n + ci) * CNN_K + k] : __float2bfloat16(0.0f);
+        }
+    }
+    for (int i = tid; i < CNN_C * CNN_K; i += NET_THREADS) w4[i] = __bfloat162float(net.w[3][i]);
+    for (int i = tid; i < 3 * CNN_C + 1; i += NET_THREADS) bias[i] = net.bias[i / CNN_C][i % CNN_C];
+    fence_proxy_async();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm = s_tmem;
+
+    uint32_t phase = 0;
+    bool failed = false;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int b = tile / tiles_per_curve;
+        const int t0 = (tile - b * tiles_per_curve) * NET_OUT;
+        // layer 0: log1p of the features, rows t0 - 16 + i
+        const float *fb = features + (int64_t)b * cin * T;
+        for (int it = tid; it < NET_XROWS * units1; it += NET_THREADS) {
+            const int u = it / NET_XROWS, i = it - u * NET_XROWS;
+            const int t = t0 - 16 + i;
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int ci = u * 8 + e;
+                v[e] = t >= 0 && t < T && ci < cin ? fb[(int64_t)ci * T + t] : 0.0f;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = log1pf(fmaxf(v[e], 0.0f));
+            if (STORE && t >= t0 && t < T && t < t0 + NET_OUT)
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    if (u * 8 + e < cin)
+                        net.act[0][((int64_t)b * cin + u * 8 + e) * T + t] = v[e];
+            net_store_row(x0 + (uint32_t)(u * NET_UNIT + i * 16), v);
+        }
+        fence_proxy_async();
+        __syncthreads();
+        for (int l = 0; l < 3; ++l) {
+            const int units = l == 0 ? units1 : 4;
+            const uint32_t wl = w0 + (l == 0 ? 0 : wsize1 + (l - 1) * net_wbytes(4));
+            if (tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (int mb = 0; mb < 2; ++mb) {
+                    for (int g = 0; g < NET_GRP; ++g) {
+                        const uint32_t d = tm + (uint32_t)((mb * NET_GRP + g) * CNN_C);
+                        const int k1 = g == NET_GRP - 1 ? CNN_K : 2 * g + 2;
+                        bool add = false;
+                        for (int q = 2; q >= 0; --q)
+                            for (int k = 2 * g; k < k1; ++k)
+                                for (int u = 0; u < units; u += 2) {
+                                    net_mma(d,
+                                            net_desc(x0 + (uint32_t)(q * NET_PART + u * NET_UNIT +
+                                                                     (mb * 128 + k) * 16),
+                                                     NET_UNIT),
+                                            net_desc(wl + (uint32_t)((k * units + u) * CNN_C * 16),
+                                                     CNN_C * 16),
+                                            add);
+                                    add = true;
+                                }
+                    }
+                    net_commit(&done[mb]);
+                }
+            }
+            __syncwarp();
+            // epilogue: warps 0-3 the rows of block 0, warps 4-7 of block 1 (in place: the other
+            // block's instructions read no row of this one). The last layer's FP32 activations
+            // overlay the parts, so it waits for both blocks.
+            const int mb = warp >> 2, r = mb * 128 + (warp & 3) * 32 + lane;
+            bool ok = mbar_wait(&done[mb], phase);
+            if (l == 2) {
+                ok = mbar_wait(&done[mb ^ 1], phase) && ok;
+                __syncthreads();
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int t = t0 - 12 + 4 * l + r;
+            const bool inside = t >= 0 && t < T;
+            const bool own = STORE && inside && t >= t0 && t < t0 + NET_OUT;
+            const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float v[16], o[16];
+                net_tmem_load(v, src + h * 16);
+                net_tmem_wait(v);
+#pragma unroll
+                for (int g = 1; g < NET_GRP; ++g) {
+                    net_tmem_load(o, src + g * CNN_C + h * 16);
+                    net_tmem_wait(o);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) v[c] += o[c];
+                }
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    const float a = fmaxf(v[c] + bias[l * CNN_C + h * 16 + c], 0.0f);
+                    v[c] = inside ? a : 0.0f;
+                }
+                if (own)
+#pragma unroll
+                    for (int c = 0; c < 16; ++c)
+                        net.act[l + 1][((int64_t)b * CNN_C + h * 16 + c) * T + t] = v[c];
+                if (l < 2) {
+                    net_store_row(x0 + (uint32_t)(2 * h * NET_UNIT + r * 16), v);
+                    net_store_row(x0 + (uint32_t)((2 * h + 1) * NET_UNIT + r * 16), v + 8);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) act3[(h * 16 + c) * NET_ACT3_LD + r] = v[c];
+                }
+            }
+            phase ^= 1u;
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            fence_proxy_async();
+            failed = __syncthreads_or(!ok);  // a wait gave up: the tile's outputs are NaN
+            if (failed) break;
+        }
+        if (failed) {
+            mbar_wait(&done[0], phase ^ 1u);  // (bounded) before the tensor memory goes
+            mbar_wait(&done[1], phase ^ 1u);
+            float *out = STORE ? net.act[CNN_LAYERS] : prob;
+            for (int o = tid; o < NET_OUT && t0 + o < T; o += NET_THREADS)
+                out[(int64_t)b * T + t0 + o] = __int_as_float(0x7fc00000);
+            break;
+        }
+        // layer 4 (one output channel, FP32): 4 bins x 8 input channels per thread
+        {
+            const int q = tid & 63, cg = tid >> 6;
+            if (q < NET_OUT / 4) {
+                float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const int ci = cg * 8 + c;
+                    float xv[12];
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        const float4 f =
+                            *reinterpret_cast<const float4 *>(&act3[ci * NET_ACT3_LD + 4 * q + 4 * m]);
+                        xv[4 * m] = f.x;
+                        xv[4 * m + 1] = f.y;
+                        xv[4 * m + 2] = f.z;
+                        xv[4 * m + 3] = f.w;
+                    }
+#pragma unroll
+                    for (int k = 0; k < CNN_K; ++k) {
+                        const float wk = w4[ci * CNN_K + k];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[e] = fmaf(wk, xv[e + k], acc[e]);
+                    }
+                }
+                *reinterpret_cast<float4 *>(&part[cg * NET_ROWS + 4 * q]) =
+                    make_float4(acc[0], acc[1], acc[2], acc[3]);
+            }
+            __syncthreads();
+            for (int o = tid; o < NET_OUT && t0 + o < T; o += NET_THREADS) {
+                const float z = (part[o] + part[NET_ROWS + o]) +
+                                (part[2 * NET_ROWS + o] + part[3 * NET_ROWS + o]) +
+                                bias[3 * CNN_C];
+                if (STORE)
+                    net.act[CNN_LAYERS][(int64_t)b * T + t0 + o] = z;
+                else
+                    prob[(int64_t)b * T + t0 + o] = 1.0f / (1.0f + expf(-z));
+            }
+            __syncthreads();  // act3 and part are read before the next tile's rows
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm),
+                     "n"(NET_TMEM_COLS));
 }
 
 // Weight and bias gradients of one conv layer:
@@ -203,12 +529,6 @@ __global__ void cnn_bce_kernel(const float *__restrict__ z, const float *__restr
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
         if (lane == 0) atomicAdd(loss, acc / (double)n);
     }
-}
-
-__global__ void cnn_sigmoid_kernel(const float *__restrict__ z, float *__restrict__ p, int64_t n) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        p[i] = 1.0f / (1.0f + expf(-z[i]));
 }
 
 __global__ void cnn_round_kernel(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wb,
@@ -369,19 +689,24 @@ cudaError_t conv(cetra_ctx *ctx, const float *x, const __nv_bfloat16 *w, const f
     return cudaGetLastError();
 }
 
-cudaError_t forward(cetra_ctx *ctx, cetra_cnn *n, const float *features, int B) {
-    const int64_t nin = (int64_t)B * n->cin * n->T;
-    cnn_prep_kernel<<<grid_for(nin, 256, ctx->num_sms), 256, 0, ctx->stream>>>(features,
-                                                                                n->d_act[0], nin);
-    ctx->launches++;
-    cudaError_t e = cudaGetLastError();
-    if (e) return e;
+// The forward pass: probabilities of B curves into prob, or (prob NULL, training) the layers'
+// activations and the logits into the network's buffers.
+cudaError_t forward(cetra_ctx *ctx, cetra_cnn *n, const float *features, int B, float *prob) {
+    net_layers net;
     for (int l = 0; l < CNN_LAYERS; ++l) {
-        e = conv(ctx, n->d_act[l], n->d_wb + n->w_off[l], n->d_params + n->b_off[l],
-                 n->d_act[l + 1], n->ch_in[l], n->ch_out[l], n->T, B, l < CNN_LAYERS - 1);
-        if (e) return e;
+        net.w[l] = n->d_wb + n->w_off[l];
+        net.bias[l] = n->d_params + n->b_off[l];
     }
-    return cudaSuccess;
+    for (int l = 0; l <= CNN_LAYERS; ++l) net.act[l] = n->d_act[l];
+    const int per = (n->T + NET_OUT - 1) / NET_OUT;
+    const int64_t tiles = (int64_t)per * B;
+    if (tiles > 2147483647) return cudaErrorInvalidConfiguration;
+    const unsigned blocks = (unsigned)std::min<int64_t>(tiles, 2 * (int64_t)ctx->num_sms);
+    auto kern = prob ? cnn_net_kernel<false> : cnn_net_kernel<true>;
+    kern<<<blocks, NET_THREADS, net_smem(n->cin), ctx->stream>>>(features, net, prob, n->cin, n->T,
+                                                               (int)tiles, per);
+    ctx->launches++;
+    return cudaGetLastError();
 }
 
 cudaError_t round_weights(cetra_ctx *ctx, cetra_cnn *n) {
@@ -458,6 +783,10 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
     e = cudaMemcpy(n->d_params, init.data(), P * 4, cudaMemcpyHostToDevice);
     if (!e) e = cudaMemset(n->d_m, 0, P * 4);
     if (!e) e = cudaMemset(n->d_v, 0, P * 4);
+    for (auto fn : {cnn_net_kernel<false>, cnn_net_kernel<true>})
+        if (!e)
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)net_smem(CNN_C));
     if (!e)
         e = cudaFuncSetAttribute(cnn_conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)conv_smem(CNN_C, CNN_C));
@@ -523,14 +852,7 @@ int cetra_cnn_forward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features, int
         return set_error(ctx, CETRA_EINVAL, "cnn_forward: bad argument");
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
-    if (!e) e = forward(ctx, n, d_features, B);
-    if (!e) {
-        const int64_t m = (int64_t)B * n->T;
-        cnn_sigmoid_kernel<<<grid_for(m, 256, ctx->num_sms), 256, 0, ctx->stream>>>(
-            n->d_act[CNN_LAYERS], d_prob, m);
-        ctx->launches++;
-        e = cudaGetLastError();
-    }
+    if (!e) e = forward(ctx, n, d_features, B, d_prob);
     return e ? cnn_fail(ctx, e, "cnn_forward") : CETRA_OK;
 }
 
@@ -542,7 +864,7 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
     const int T = n->T;
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
-    if (!e) e = forward(ctx, n, d_features, B);
+    if (!e) e = forward(ctx, n, d_features, B, nullptr);
     if (!e) e = cudaMemsetAsync(n->d_grads, 0, (size_t)n->n_params * 4, ctx->stream);
     if (!e) e = cudaMemsetAsync(n->d_loss, 0, sizeof(double), ctx->stream);
     const int64_t m = (int64_t)B * T;
