@@ -23,21 +23,43 @@ namespace {
 
 
 // --------------------------------------------------------------------------------------------
+// floor((t - t_ref) / c + 1/2), each operation rounded once (Sec. 2.1.1): the nearest grid point
+// of time t. What bounds the resampling is FP64 (2 lanes per clock and SM), and half of that was
+// the division: x = (t - t_ref) (1 / c) is within 2^-20 of the quotient while |x| < 2^31, so the
+// nearest integer of x is the answer unless x lies within 2^-19 of a half-integer, where the
+// division decides. (x + 1.5 2^52 has the nearest integer in its low bits.)
+__device__ __forceinline__ bool grid_point(double t, double t_ref, double c, double rc,
+                                           int64_t n_pad, int64_t n_grid, int64_t &bin) {
+    const double d = __dsub_rn(t, t_ref);
+    const double x = __dmul_rn(d, rc);
+    const double z = __dadd_rn(x, 6755399441055744.0);
+    const double f = __dsub_rn(x, __dsub_rn(z, 6755399441055744.0));
+    // high words of 2^31 and of 1/2 - 2^-19
+    if ((uint32_t)(__double2hiint(x) & 0x7fffffff) < 0x41e00000u &&
+        (uint32_t)(__double2hiint(f) & 0x7fffffff) < 0x3fdffff8u) {
+        bin = n_pad + (int64_t)__double2loint(z);
+        return bin >= 0 && bin < n_grid;  // else outside the planned grid
+    }
+    const double v = floor(__dadd_rn(__ddiv_rn(d, c), 0.5));
+    if (!(v >= -(double)n_pad) || !(v < (double)(n_grid - n_pad))) return false;
+    bin = n_pad + (int64_t)v;
+    return true;
+}
+
 // Sec. 2.1.1: each observation goes to the nearest grid point
 // k = n_pad + floor((t - t_ref) / c + 1/2) and accumulates W = 1/sigma^2 and W y.
 __global__ void resample_kernel(const double *__restrict__ time, const float *__restrict__ flux,
                                 const float *__restrict__ err, int64_t n, double t_ref, double c,
-                                int64_t n_pad, int64_t n_grid, int flux_is_offset,
+                                double rc, int64_t n_pad, int64_t n_grid, int flux_is_offset,
                                 float2 *__restrict__ grid) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
         const double tk = time[k];
         const float fk = flux[k], ek = err[k];
         if (!(isfinite(tk) && isfinite(fk) && isfinite(ek) && ek > 0.0f)) continue;
-        const double v = floor(__dadd_rn(__ddiv_rn(__dsub_rn(tk, t_ref), c), 0.5));
         // drop points outside the planned grid (a curve that does not match its plan)
-        if (!(v >= -(double)n_pad) || !(v < (double)(n_grid - n_pad))) continue;
-        const int64_t bin = n_pad + (int64_t)v;
+        int64_t bin;
+        if (!grid_point(tk, t_ref, c, rc, n_pad, n_grid, bin)) continue;
         const float wk = 1.0f / (ek * ek);
         const float yk = flux_is_offset ? fk : 1.0f - fk;
         atomicAdd(&grid[bin], make_float2(wk * yk, wk));  // (W y, W), one cell
@@ -256,6 +278,48 @@ linear_kernel(const float2 *__restrict__ grid, int64_t n_grid,
 
 // --------------------------------------------------------------------------------------------
 // Sec. 2.3: the per-period winner, re-summed in FP64 from the FP32 grid.
+//
+// A winner's sum is a chain of dependent FP64 adds behind loads whose addresses take FP64
+// arithmetic too; with a thread per period the longest chain (one term per epoch) was the
+// kernel's time whatever the number of periods (38 us at 2,000 periods and 54 epochs). FIN_LANES
+// neighbouring lanes now share a winner, each with FIN_CHAINS sums in flight: chain m of lane l
+// adds epochs l + FIN_LANES m, + FIN_LANES FIN_CHAINS, ..., and the chains' and lanes' sums are
+// added in pairs (every caller the same way, so that equal models stay equal). More lanes would
+// cost large grids their FP64 rate (2 lanes per clock and SM).
+constexpr int FIN_LANES = 8;
+constexpr int FIN_CHAINS = 4;
+
+// (sum A, sum B) over the epochs of t0 index i of a period of Ps t0 steps, in every lane of the
+// group; sub = the lane's place in it.
+__device__ __forceinline__ void winner_sums(const float2 *__restrict__ row, int64_t i, int64_t I,
+                                            double Ps, int sub, double &SA, double &SB) {
+    double a[FIN_CHAINS], b[FIN_CHAINS];
+#pragma unroll
+    for (int m = 0; m < FIN_CHAINS; ++m) a[m] = b[m] = 0.0;
+    bool more = true;
+    for (int64_t e = sub; more; e += FIN_LANES * FIN_CHAINS) {
+        float2 v[FIN_CHAINS];
+#pragma unroll
+        for (int m = 0; m < FIN_CHAINS; ++m) {
+            const int64_t cell = i + epoch_offset(e + m * FIN_LANES, Ps);
+            more = cell < I;  // the offsets grow with e
+            v[m] = more ? row[cell] : make_float2(0.0f, 0.0f);
+        }
+#pragma unroll
+        for (int m = 0; m < FIN_CHAINS; ++m) {
+            a[m] = __dadd_rn(a[m], (double)v[m].x);
+            b[m] = __dadd_rn(b[m], (double)v[m].y);
+        }
+    }
+    SA = __dadd_rn(__dadd_rn(a[0], a[1]), __dadd_rn(a[2], a[3]));
+    SB = __dadd_rn(__dadd_rn(b[0], b[1]), __dadd_rn(b[2], b[3]));
+#pragma unroll
+    for (int o = 1; o < FIN_LANES; o <<= 1) {
+        SA = __dadd_rn(SA, __shfl_xor_sync(0xFFFFFFFFu, SA, o));
+        SB = __dadd_rn(SB, __shfl_xor_sync(0xFFFFFFFFu, SB, o));
+    }
+}
+
 __global__ void finalize_kernel(const float2 *__restrict__ ab, int64_t I, int64_t ld,
                                 const double *__restrict__ durations,
                                 const double *__restrict__ periods, int K,
@@ -263,41 +327,30 @@ __global__ void finalize_kernel(const float2 *__restrict__ ab, int64_t I, int64_
                                 const int *__restrict__ status, double t_ref, double c,
                                 int64_t p, int64_t q, int64_t n_pad, double *dlogl, double *t0,
                                 double *dur, double *depth, double *var, int64_t *oi, int32_t *oj) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= K) return;
-    const unsigned long long key = keys[k];
+    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t k = x / FIN_LANES;
+    const int sub = (int)(x % FIN_LANES);
+    const unsigned long long key = k < K ? keys[k] : 0ull;
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    if (key == 0ull || *status != 0) {  // null period, or the fold gave up
-        if (dlogl) dlogl[k] = nan;
-        if (t0) t0[k] = nan;
-        if (dur) dur[k] = nan;
-        if (depth) depth[k] = nan;
-        if (var) var[k] = nan;
-        if (oi) oi[k] = -1;
-        if (oj) oj[k] = -1;
-        return;
-    }
+    const bool found = key != 0ull && *status == 0;  // else a null period, or the fold gave up
     const uint32_t flat = 0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull);
-    const int64_t j = (int64_t)flat / I, i = (int64_t)flat % I;
-    const double Ps = period_steps(periods[k], c, p, q);
-    const float2 *row = ab + j * ld;
-    double SA = 0.0, SB = 0.0;
-    for (int64_t e = 0;; ++e) {
-        const int64_t cell = i + epoch_offset(e, Ps);
-        if (cell >= I) break;
-        const float2 v = row[cell];
-        SA = __dadd_rn(SA, (double)v.x);
-        SB = __dadd_rn(SB, (double)v.y);
-    }
+    const uint32_t j = found ? flat / (uint32_t)I : 0u;
+    const int64_t i = found ? (int64_t)(flat - j * (uint32_t)I) : I;  // I: no epoch
+    double SA, SB;
+    winner_sums(ab + (int64_t)j * ld, i, I,
+                found ? period_steps(periods[k], c, p, q) : 1.0, sub, SA, SB);
+    if (k >= K || sub != 0) return;
     const double Z = __ddiv_rn(SA, SB);
-    if (dlogl) dlogl[k] = 0.5 * __dmul_rn(SA, Z);
-    if (depth) depth[k] = Z;
-    if (var) var[k] = __ddiv_rn(1.0, SB);
+    if (dlogl) dlogl[k] = found ? 0.5 * __dmul_rn(SA, Z) : nan;
+    if (depth) depth[k] = found ? Z : nan;
+    if (var) var[k] = found ? __ddiv_rn(1.0, SB) : nan;
     if (t0)
-        t0[k] = __dadd_rn(t_ref, __ddiv_rn(__dmul_rn((double)(i * p - n_pad * q), c), (double)q));
-    if (dur) dur[k] = durations[j];
-    if (oi) oi[k] = i;
-    if (oj) oj[k] = (int32_t)j;
+        t0[k] = found ? __dadd_rn(t_ref, __ddiv_rn(__dmul_rn((double)(i * p - n_pad * q), c),
+                                                   (double)q))
+                      : nan;
+    if (dur) dur[k] = found ? durations[j] : nan;
+    if (oi) oi[k] = found ? i : -1;
+    if (oj) oj[k] = found ? (int32_t)j : -1;
 }
 
 // --------------------------------------------------------------------------------------------
@@ -338,7 +391,7 @@ __global__ void batch_resample_kernel(const double *__restrict__ time,
                                       const float *__restrict__ err, int64_t n,
                                       const int64_t *__restrict__ pt_off, int n_curves,
                                       const batch_curve *__restrict__ curves, double c,
-                                      int64_t n_pad, int flux_is_offset,
+                                      double rc, int64_t n_pad, int flux_is_offset,
                                       float2 *__restrict__ grid) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
@@ -346,9 +399,9 @@ __global__ void batch_resample_kernel(const double *__restrict__ time,
         const float fk = flux[k], ek = err[k];
         if (!(isfinite(tk) && isfinite(fk) && isfinite(ek) && ek > 0.0f)) continue;
         const batch_curve cv = curves[csr_find(pt_off, n_curves, k)];
-        const double v = floor(__dadd_rn(__ddiv_rn(__dsub_rn(tk, cv.t_ref), c), 0.5));
-        if (!(v >= -(double)n_pad) || !(v < (double)((int64_t)cv.n_grid - n_pad))) continue;
-        const int64_t bin = cv.grid_off + n_pad + (int64_t)v;
+        int64_t bin;
+        if (!grid_point(tk, cv.t_ref, c, rc, n_pad, cv.n_grid, bin)) continue;
+        bin += cv.grid_off;
         const float wk = 1.0f / (ek * ek);
         const float yk = flux_is_offset ? fk : 1.0f - fk;
         atomicAdd(&grid[bin], make_float2(wk * yk, wk));
@@ -389,33 +442,37 @@ __global__ void batch_finalize_kernel(const float2 *__restrict__ ab,
                                       const unsigned long long *__restrict__ curve_keys,
                                       const int *__restrict__ status,
                                       cetra_best *__restrict__ best) {
-    const int cidx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (cidx >= n_curves) return;
+    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int sub = (int)(x % FIN_LANES);
+    const bool present = x / FIN_LANES < n_curves;
+    const int cidx = present ? (int)(x / FIN_LANES) : 0;
     const batch_curve cv = curves[cidx];
-    const unsigned long long key = curve_keys[cidx];
+    const unsigned long long key = present ? curve_keys[cidx] : 0ull;
+    const bool found = key != 0ull && *status == 0;
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     cetra_best out;
     out.dlogl = out.period = out.t0 = out.duration = out.depth = out.depth_var = nan;
     out.k = out.i = -1;
     out.j = -1;
     out.n_periods = cv.n_periods;
-    if (key == 0ull || *status != 0) {
+    int64_t k = 0;
+    int j = 0, i = cv.I;  // i = I: no epoch
+    double P = 0.0;
+    if (found) {
+        k = (int64_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
+        const unsigned long long pk = period_keys[cv.per_off + k];
+        const uint32_t flat = 0xFFFFFFFFu - (uint32_t)(pk & 0xFFFFFFFFull);
+        j = (int)(flat / (uint32_t)cv.I);
+        i = (int)(flat % (uint32_t)cv.I);
+        P = batch_period(cv.pmin, cv.ratio, k);
+    }
+    double SA, SB;
+    winner_sums(ab + cv.ab_off + (int64_t)j * cv.ld, i, cv.I,
+                found ? period_steps(P, c, p, q) : 1.0, sub, SA, SB);
+    if (!present || sub != 0) return;
+    if (!found) {
         best[cidx] = out;
         return;
-    }
-    const int64_t k = (int64_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
-    const unsigned long long pk = period_keys[cv.per_off + k];
-    const uint32_t flat = 0xFFFFFFFFu - (uint32_t)(pk & 0xFFFFFFFFull);
-    const int j = (int)(flat / (uint32_t)cv.I), i = (int)(flat % (uint32_t)cv.I);
-    const double P = batch_period(cv.pmin, cv.ratio, k);
-    const double Ps = period_steps(P, c, p, q);
-    const float2 *row = ab + cv.ab_off + (int64_t)j * cv.ld;
-    double SA = 0.0, SB = 0.0;
-    for (int64_t e = 0;; ++e) {
-        const int64_t cell = i + epoch_offset(e, Ps);
-        if (cell >= cv.I) break;
-        SA = __dadd_rn(SA, (double)row[cell].x);
-        SB = __dadd_rn(SB, (double)row[cell].y);
     }
     const double Z = __ddiv_rn(SA, SB);
     out.dlogl = 0.5 * __dmul_rn(SA, Z);
@@ -643,7 +700,8 @@ cudaError_t launch_resample(cetra_ctx *ctx, const cetra_plan *plan, const double
     blocks = blocks > (int64_t)ctx->num_sms * 16 ? (int64_t)ctx->num_sms * 16 : blocks;
     prof_mark(ctx, KID_RESAMPLE, true);
     resample_kernel<<<(unsigned)blocks, threads, 0, ctx->stream>>>(
-        time, flux, err, n, plan->t_ref, plan->cadence, plan->n_pad, plan->n_grid,
+        time, flux, err, n, plan->t_ref, plan->cadence, 1.0 / plan->cadence, plan->n_pad,
+        plan->n_grid,
         plan->flux_is_offset, grid);
     prof_mark(ctx, KID_RESAMPLE, false);
     ctx->launches++;
@@ -706,9 +764,10 @@ cudaError_t launch_finalize(cetra_ctx *ctx, const cetra_plan *plan, const float2
                             const int *status, double *dlogl, double *t0, double *dur, double *depth, double *var,
                             int64_t *oi, int32_t *oj) {
     if (K <= 0) return cudaSuccess;
-    const int threads = 128;
+    const int threads = 32;  // small grids reach more SMs' FP64 pipes
     prof_mark(ctx, KID_FINALIZE, true);
-    finalize_kernel<<<(K + threads - 1) / threads, threads, 0, ctx->stream>>>(
+    const int64_t lanes = (int64_t)K * FIN_LANES;
+    finalize_kernel<<<(unsigned)((lanes + threads - 1) / threads), threads, 0, ctx->stream>>>(
         ab, plan->n_t0, plan->ab_ld, plan->d_durations, periods, K, keys, status, plan->t_ref,
         plan->cadence, plan->p,
         plan->q, plan->n_pad, dlogl, t0, dur, depth, var, oi, oj);
@@ -753,7 +812,8 @@ cudaError_t launch_batch_resample(cudaStream_t stream, int num_sms, const cetra_
     int64_t blocks = (n_points + threads - 1) / threads;
     if (blocks > (int64_t)num_sms * 32) blocks = (int64_t)num_sms * 32;
     batch_resample_kernel<<<(unsigned)blocks, threads, 0, stream>>>(
-        time, flux, err, n_points, pt_offsets, n_curves, curves, plan->cadence, plan->n_pad,
+        time, flux, err, n_points, pt_offsets, n_curves, curves, plan->cadence,
+        1.0 / plan->cadence, plan->n_pad,
         plan->flux_is_offset, grid);
     return cudaGetLastError();
 }
@@ -783,7 +843,8 @@ cudaError_t launch_batch_finalize(cudaStream_t stream, const cetra_plan *plan, c
                                   cetra_best *best) {
     if (n_curves <= 0) return cudaSuccess;
     const int threads = 128;
-    batch_finalize_kernel<<<(n_curves + threads - 1) / threads, threads, 0, stream>>>(
+    const int64_t lanes = (int64_t)n_curves * FIN_LANES;
+    batch_finalize_kernel<<<(unsigned)((lanes + threads - 1) / threads), threads, 0, stream>>>(
         ab, curves, n_curves, plan->d_durations, plan->cadence, plan->p, plan->q, plan->n_pad,
         period_keys, curve_keys, status, best);
     return cudaGetLastError();

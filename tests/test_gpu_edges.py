@@ -1,0 +1,77 @@
+"""Kernel variants at the sizes where they can go wrong, against the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import cnn as ocnn
+from _parity import compare_linear, gpu_search, oracle_search
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("offset", [0.0, 2.45e6])
+def test_resample_at_half_points(offset):
+    """Times within a few ulps of the midpoint between two grid points: the nearest point is
+    decided by the FP64 division, and its reciprocal shortcut must not decide otherwise."""
+    c = 120.0 / 86400.0
+    k = np.arange(600)
+    t = offset + k * c
+    half = (k % 3) == 1
+    t[half] = offset + (k[half] + 0.5) * c
+    for u in range(4):  # 0, 1, 2, 3 ulps either side
+        sel = half & (k % 4 == u)
+        for _ in range(u):
+            t[sel] = np.nextafter(t[sel], np.where(k[sel] % 8 < 4, np.inf, -np.inf))
+    rng = np.random.default_rng(3)
+    f = (1.0 + rng.normal(0.0, 1e-3, t.size)).astype(np.float32)
+    e = np.full(t.size, 1e-3, np.float32)
+    d = np.array([0.03, 0.1])
+    tm = np.ones(64, np.float32)
+    kw = dict(cadence=c, t0_step=c)
+    compare_linear(gpu_search(t, f, e, d, tm, **kw), oracle_search(t, f, e, d, tm, **kw), d)
+
+
+@pytest.mark.parametrize("T,bin_days,valid,lo,hi,n", [
+    (256, 0.4, 256, 0.5, 0.56, 2),       # 2 phases: eight trials share a warp
+    (256, 0.1, 256, 0.7, 0.74, 2),       # 8 phases: four trials
+    (256, 0.1, 231, 1.5, 1.58, 3),       # 16 phases: two trials
+    (256, 0.02, 255, 0.6, 0.65, 2),      # 31 to 33 phases: one and two rows
+    (1024, 0.01, 1001, 1.27, 1.29, 2),   # 127 to 129 phases: four and five rows
+    (1024, 0.01, 1024, 3.5, 3.53, 2),    # 350 phases: 12 rows, of which 11 hold phases
+    (1536, 0.01, 1536, 7.6, 7.68, 2),    # 768 phases: two units, two epochs
+    (25088, 0.002, 1200, 0.6, 0.61, 1),  # a map that is not staged in shared memory
+])
+def test_comb_shapes(T, bin_days, valid, lo, hi, n):
+    """Scores over the shapes the comb's lanes take; the sums are of at most 256 terms, each
+    rounded once (relative error below 256 * 2^-24 = 1.6e-5, far less for random signs)."""
+    import torch
+    from paper_2503_20875_gb300 import Context, cetra_cnn_comb
+    rng = np.random.default_rng(T)
+    m = (rng.uniform(size=(3, T)) ** 6).astype(np.float32)
+    bw = np.array([bin_days, bin_days * 1.1, bin_days])
+    nv = np.array([valid, valid, valid // 2], np.int32)
+    scores = torch.empty((3, n), dtype=torch.float32, device="cuda")
+    cetra_cnn_comb(Context(0), torch.from_numpy(m).cuda(), torch.from_numpy(bw).cuda(), lo, hi, n,
+                   scores, torch.from_numpy(nv).cuda())
+    np.testing.assert_allclose(scores.cpu().numpy(), ocnn.comb(m, bw, lo, hi, n, nv), rtol=1.6e-5,
+                               atol=1e-7)
+
+
+@pytest.mark.parametrize("cin,T,B", [(1, 256, 1), (16, 256, 3), (17, 512, 2), (32, 768, 2)])
+def test_network_tiles(cin, T, B):
+    """Probabilities over channel counts that fill one and two K steps, one to four tiles per
+    curve, a ragged last tile, zero padding at both ends and large inputs. Tolerance: 288 products
+    per sum and layer, as in the network's parity test."""
+    import torch
+    from paper_2503_20875_gb300 import CNN, Context
+    rng = np.random.default_rng(cin + T)
+    f = (rng.chisquare(1, (B, cin, T)) * 3.0).astype(np.float32)
+    f[0, 0, :5] = 1e4
+    f[-1, -1, -3:] = 3e7
+    net = CNN(Context(0), cin, n_bins=T, max_batch=B, seed=cin)
+    p = net.get_params()
+    p += rng.normal(0.0, 0.01, p.size).astype(np.float32)  # biases too
+    net.set_params(p)
+    out = torch.empty((B, T), dtype=torch.float32, device="cuda")
+    net.forward(torch.from_numpy(f).cuda(), out)
+    np.testing.assert_allclose(out.cpu().numpy(), ocnn.probabilities(p, f), rtol=0, atol=2e-5)
