@@ -3,6 +3,7 @@
 //    around the signal's transits are nulled, then the linear stage is rerun;
 //  - single-transit (monotransit) events from the linear search (Sec. 1, Sec. 5): the
 //    strongest dimming windows, greedily, each hiding the mid-times within its duration.
+#include <algorithm>
 #include <cmath>
 
 #include "internal.h"
@@ -41,73 +42,137 @@ __device__ __forceinline__ unsigned long long event_key(float lr, int j, int64_t
            ((unsigned long long)(255 - j) << 24) | (unsigned long long)(0xFFFFFF - i);
 }
 
-__global__ void mono_keys_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I, int J,
-                                 unsigned long long *__restrict__ keys) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < I; i += stride) {
-        unsigned long long best = 0ull;
-        for (int j = 0; j < J; ++j) {
-            const float2 v = ab[(int64_t)j * ld + i];
-            if (v.y > 0.0f && v.x > 0.0f) {
-                const float lr = 0.5f * (v.x * (v.x / v.y));
-                if (lr > 0.0f) best = max(best, event_key(lr, j, i));
-            }
-        }
-        keys[i] = best;
-    }
+// The greedy steps are serial and short, so what bounded them was two launches a step, the first
+// a pass over every key (12 us a step at 2.1 M t0 cells). The keys are now kept with the best of
+// each segment of 2^shift cells (at most EV_SEGMENTS), and one block takes all the steps: it
+// scans the segments' maxima in shared memory, and after a step works out again only those of the
+// segments that the event hides cells of.
+constexpr int EV_THREADS = 1024;
+constexpr int EV_SEGMENTS = 4096;
+__host__ __device__ inline int event_shift(int64_t I) {
+    int shift = 8;
+    while (((I + ((int64_t)1 << shift) - 1) >> shift) > EV_SEGMENTS) ++shift;
+    return shift;
 }
 
-// Greedy step e: the best key left (the cells earlier events hide have key 0). Nothing to do
-// once a previous step found nothing.
-__global__ void mono_pick_kernel(const unsigned long long *__restrict__ keys, int64_t I, int e,
-                                 unsigned long long *__restrict__ slots) {
-    if (e > 0 && slots[e - 1] == 0ull) return;  // uniform
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
+    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    return v;
+}
+
+// One block per segment: the keys of its cells and their maximum.
+__global__ void __launch_bounds__(NB_THREADS)
+mono_keys_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I, int J, int shift,
+                 unsigned long long *__restrict__ keys, unsigned long long *__restrict__ top) {
     __shared__ unsigned long long red[NB_THREADS / 32];
-    unsigned long long best = 0ull;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < I; i += stride)
-        best = max(best, keys[i]);
-    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_down_sync(0xFFFFFFFFu, best, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
+    const int64_t lo = (int64_t)blockIdx.x << shift;
+    const int64_t hi = min(I, lo + ((int64_t)1 << shift));
+    unsigned long long most = 0ull;
+    auto take = [](float x, float y, int j, int64_t i, unsigned long long &best) {
+        if (y > 0.0f && x > 0.0f) {
+            const float lr = 0.5f * (x * (x / y));
+            if (lr > 0.0f) best = max(best, event_key(lr, j, i));
+        }
+    };
+    // two cells per load (the rows' strides and a segment's first cell are even; the row goes on
+    // after its last cell)
+    for (int64_t i = lo + 2 * threadIdx.x; i < hi; i += 2 * NB_THREADS) {
+        unsigned long long best0 = 0ull, best1 = 0ull;
+#pragma unroll 4
+        for (int j = 0; j < J; ++j) {
+            const float4 v = *reinterpret_cast<const float4 *>(ab + (int64_t)j * ld + i);
+            take(v.x, v.y, j, i, best0);
+            take(v.z, v.w, j, i + 1, best1);
+        }
+        keys[i] = best0;
+        if (i + 1 < hi)
+            keys[i + 1] = best1;
+        else
+            best1 = 0ull;
+        most = max(most, max(best0, best1));
+    }
+    most = warp_max(most);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = most;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int x = 1; x < NB_THREADS / 32; ++x) best = max(best, red[x]);
-        if (best) atomicMax(&slots[e], best);
+        for (int x = 1; x < NB_THREADS / 32; ++x) most = max(most, red[x]);
+        top[blockIdx.x] = most;
     }
 }
 
-// Decode step e's key into event e (FP64 values from the window's FP32 sums), then hide the
-// t0 cells within its duration: |i - i_e| < h = D_j q / (c p) (FP64) -> key 0. One block.
-__global__ void __launch_bounds__(NB_THREADS)
-mono_event_kernel(const unsigned long long *__restrict__ slots, int e,
-                  const float2 *__restrict__ ab, int64_t ld, int64_t I,
-                  const double *__restrict__ durations, double t_ref, double c, int64_t p,
-                  int64_t q, int64_t n_pad, unsigned long long *__restrict__ keys,
-                  cetra_event *__restrict__ events, int *__restrict__ n_events) {
-    const unsigned long long key = slots[e];
-    if (key == 0ull || (e > 0 && slots[e - 1] == 0ull)) return;  // uniform
-    const int64_t ie = 0xFFFFFF - (int64_t)(key & 0xFFFFFFull);
-    const int j = 255 - (int)((key >> 24) & 0xFFull);
-    const double h = __ddiv_rn(__dmul_rn(durations[j], (double)q), __dmul_rn(c, (double)p));
-    if (threadIdx.x == 0) {
-        const float2 v = ab[(int64_t)j * ld + ie];
-        cetra_event ev;
-        ev.depth = __ddiv_rn((double)v.x, (double)v.y);
-        ev.depth_var = __ddiv_rn(1.0, (double)v.y);
-        ev.dlogl = 0.5 * __dmul_rn((double)v.x, ev.depth);
-        ev.t0 = __dadd_rn(t_ref, __ddiv_rn(__dmul_rn((double)(ie * p - n_pad * q), c), (double)q));
-        ev.duration = durations[j];
-        ev.i = ie;
-        ev.j = j;
-        ev.pad_ = 0;
-        events[e] = ev;
-        *n_events = e + 1;
+// All greedy steps (one block): the best key left becomes the next event (FP64 values from the
+// window's FP32 sums), then the t0 cells within its duration are hidden: |i - i_e| < h =
+// D_j q / (c p) (FP64) -> key 0. Ends early when no key is left.
+__global__ void __launch_bounds__(EV_THREADS)
+mono_events_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I,
+                   const double *__restrict__ durations, double t_ref, double c, int64_t p,
+                   int64_t q, int64_t n_pad, int shift, int max_events,
+                   unsigned long long *__restrict__ keys,
+                   const unsigned long long *__restrict__ top, cetra_event *__restrict__ events,
+                   int *__restrict__ n_events) {
+    __shared__ unsigned long long seg[EV_SEGMENTS];
+    __shared__ unsigned long long red[EV_THREADS / 32];
+    __shared__ unsigned long long s_key;
+    __shared__ int64_t s_reach;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int n_seg = (int)((I + ((int64_t)1 << shift) - 1) >> shift);
+    for (int x = t; x < n_seg; x += EV_THREADS) seg[x] = top[x];
+    __syncthreads();
+    int e = 0;
+    for (; e < max_events; ++e) {
+        unsigned long long best = 0ull;
+        for (int x = t; x < n_seg; x += EV_THREADS) best = max(best, seg[x]);
+        best = warp_max(best);
+        if (lane == 0) red[wid] = best;
+        __syncthreads();
+        if (wid == 0) {
+            best = warp_max(red[lane]);
+            if (lane == 0) s_key = best;
+        }
+        __syncthreads();
+        const unsigned long long key = s_key;
+        if (key == 0ull) break;  // uniform
+        const int64_t ie = 0xFFFFFF - (int64_t)(key & 0xFFFFFFull);
+        const int j = 255 - (int)((key >> 24) & 0xFFull);
+        if (t == 0) {
+            // (one lane: FP64 in all warps would take longer than the rest of the step)
+            // integers below h are those below ceil(h)
+            const double h =
+                __ddiv_rn(__dmul_rn(durations[j], (double)q), __dmul_rn(c, (double)p));
+            const double span = ceil(h);
+            s_reach = span < (double)I ? (int64_t)span : I;
+            const float2 v = ab[(int64_t)j * ld + ie];
+            cetra_event ev;
+            ev.depth = __ddiv_rn((double)v.x, (double)v.y);
+            ev.depth_var = __ddiv_rn(1.0, (double)v.y);
+            ev.dlogl = 0.5 * __dmul_rn((double)v.x, ev.depth);
+            ev.t0 =
+                __dadd_rn(t_ref, __ddiv_rn(__dmul_rn((double)(ie * p - n_pad * q), c), (double)q));
+            ev.duration = durations[j];
+            ev.i = ie;
+            ev.j = j;
+            ev.pad_ = 0;
+            events[e] = ev;
+        }
+        __syncthreads();
+        const int64_t r = s_reach;
+        const int64_t lo = max((int64_t)0, ie - r), hi = min(I - 1, ie + r);
+        // hide the cells, and work out the maxima of their segments again (32 consecutive cells
+        // are of one segment)
+        const int64_t s0 = lo >> shift, s1 = hi >> shift;
+        for (int64_t x = s0 + t; x <= s1; x += EV_THREADS) seg[x] = 0ull;
+        __syncthreads();
+        const int64_t end = min(I, (s1 + 1) << shift);
+        for (int64_t i0 = s0 << shift; i0 < end; i0 += EV_THREADS) {
+            const int64_t i = i0 + t;
+            unsigned long long k = i < end ? keys[i] : 0ull;
+            if (k && llabs(i - ie) < r) keys[i] = k = 0ull;
+            k = warp_max(k);
+            if (lane == 0 && k) atomicMax(&seg[i >> shift], k);
+        }
+        __syncthreads();
     }
-    const double span = ceil(h);
-    const int64_t r = span < (double)I ? (int64_t)span : I;
-    const int64_t lo = max((int64_t)0, ie - r), hi = min(I - 1, ie + r);
-    for (int64_t i = lo + threadIdx.x; i <= hi; i += blockDim.x)
-        if ((double)llabs(i - ie) < h) keys[i] = 0ull;
+    if (t == 0) *n_events = e;
 }
 
 unsigned blocks_for(int64_t n, int num_sms) {
@@ -127,29 +192,24 @@ cudaError_t launch_mask(cetra_ctx *ctx, const cetra_plan *plan, float2 *grid, do
 }
 
 size_t mono_scratch_words(const cetra_plan *plan, int max_events) {
-    return (size_t)plan->n_t0 + (size_t)max_events;
+    return (size_t)plan->n_t0 + (size_t)std::max(max_events, EV_SEGMENTS);
 }
 
 cudaError_t launch_monotransits(cetra_ctx *ctx, const cetra_plan *plan, const float2 *ab,
                                 unsigned long long *scratch, int max_events,
                                 cetra_event *events, int *n_events) {
     const int64_t I = plan->n_t0;
-    unsigned long long *keys = scratch, *slots = scratch + I;
-    cudaError_t e = cudaMemsetAsync(slots, 0, (size_t)max_events * sizeof(unsigned long long),
-                                    ctx->stream);
-    if (!e) e = cudaMemsetAsync(n_events, 0, sizeof(int), ctx->stream);
-    if (e) return e;
-    const unsigned blocks = blocks_for(I, ctx->num_sms);
-    mono_keys_kernel<<<blocks, NB_THREADS, 0, ctx->stream>>>(ab, plan->ab_ld, I, plan->J, keys);
+    unsigned long long *keys = scratch, *top = scratch + I;
+    const int shift = event_shift(I);
+    const unsigned segments = (unsigned)((I + ((int64_t)1 << shift) - 1) >> shift);
+    mono_keys_kernel<<<segments, NB_THREADS, 0, ctx->stream>>>(ab, plan->ab_ld, I, plan->J, shift,
+                                                               keys, top);
     ctx->launches++;
-    if ((e = cudaGetLastError())) return e;
-    for (int m = 0; m < max_events; ++m) {
-        mono_pick_kernel<<<blocks, NB_THREADS, 0, ctx->stream>>>(keys, I, m, slots);
-        mono_event_kernel<<<1, NB_THREADS, 0, ctx->stream>>>(
-            slots, m, ab, plan->ab_ld, I, plan->d_durations, plan->t_ref, plan->cadence, plan->p,
-            plan->q, plan->n_pad, keys, events, n_events);
-        ctx->launches += 2;
-        if ((e = cudaGetLastError())) return e;
-    }
-    return cudaSuccess;
+    cudaError_t e = cudaGetLastError();
+    if (e) return e;
+    mono_events_kernel<<<1, EV_THREADS, 0, ctx->stream>>>(
+        ab, plan->ab_ld, I, plan->d_durations, plan->t_ref, plan->cadence, plan->p, plan->q,
+        plan->n_pad, shift, max_events, keys, top, events, n_events);
+    ctx->launches++;
+    return cudaGetLastError();
 }
