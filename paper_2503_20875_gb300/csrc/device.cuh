@@ -70,7 +70,7 @@ __device__ __forceinline__ void kahan_add2(float2 &s, float2 &nc, float2 v) {
 
 // Nearest epoch cell offset o_e = floor(e Ps + 1/2), FP64, no contraction.
 __device__ __forceinline__ int64_t epoch_offset(int64_t e, double Ps) {
-    return (int64_t)floor(__dadd_rn(__dmul_rn((double)e, Ps), 0.5));
+    return __double2ll_rd(__dadd_rn(__dmul_rn((double)e, Ps), 0.5));
 }
 
 // Period in t0 steps, Ps = (P q) / (c p), FP64, no contraction.

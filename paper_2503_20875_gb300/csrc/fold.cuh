@@ -219,16 +219,17 @@ struct epoch_offsets {
 };
 
 // Bit gg set when period g0 + gg is folded at duration j: it has epochs, D_j < P (Sec. 2.3)
-// and the caller's mask allows the pair.
+// and the caller's mask allows the pair. (Positive doubles order like their bits: the comparison
+// is an integer one, since every FP64 instruction of a warp takes the SM's FP64 pipe 16 clocks.)
 template <int GS>
 __device__ __forceinline__ unsigned period_use(const fold_smem &sm, int g0, int j) {
-    const double D = sm.it.durations[j];
+    const long long D = __double_as_longlong(sm.it.durations[j]);
     const uint8_t *mask = sm.it.mask;
     unsigned use = 0u;
 #pragma unroll
     for (int gg = 0; gg < GS; ++gg) {
         const int g = g0 + gg;
-        if (sm.E[g] > 0 && D < sm.P[g] &&
+        if (sm.E[g] > 0 && D < __double_as_longlong(sm.P[g]) &&
             (!mask || mask[(int64_t)(sm.it.mask_k0 + g) * sm.it.J + j]))
             use |= 1u << gg;
     }
