@@ -26,75 +26,9 @@ constexpr int CNN_K = 9;           // kernel width
 constexpr int CNN_HALF = CNN_K / 2;
 constexpr int CNN_C = 32;          // hidden channels
 constexpr int CNN_LAYERS = 4;
-constexpr int CONV_TT = 256;       // time bins per block
-constexpr int CONV_RT = 8;         // time bins per thread
-constexpr int CONV_RC = 8;         // output channels per thread
-constexpr int CONV_THREADS = (CONV_TT / CONV_RT) * (CNN_C / CONV_RC);  // 128
 constexpr size_t kCombSmemMax = 98 * 1024;  // maps up to 24,576 bins (+ 512 cells) are staged
 
 // ------------------------------------------------------------------------------- kernels
-
-// y[b][co][t] = act(bias[co] + sum_ci sum_k w[co][ci][k] x[b][ci][t + k - 4]), zero padding.
-// One block: all output channels (cout <= 32) of CONV_TT bins of one curve. Thread:
-// CONV_RT consecutive bins x CONV_RC channels; the input window slides through registers
-// and each (ci, k) weight is one broadcast shared load for CONV_RT FMAs.
-__global__ void __launch_bounds__(CONV_THREADS)
-cnn_conv_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w,
-                const float *__restrict__ bias, float *__restrict__ y, int cin, int cout, int T,
-                int relu) {
-    extern __shared__ float cs[];
-    float *ws = cs;                                // [cout][cin][9]
-    float *xs = cs + cout * cin * CNN_K;           // [cin][CONV_TT + 8]
-    const int b = blockIdx.y;
-    const int t0 = blockIdx.x * CONV_TT;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < cout * cin * CNN_K; i += blockDim.x) ws[i] = __bfloat162float(w[i]);
-    const int span = CONV_TT + CNN_K - 1;
-    const float *xb = x + (int64_t)b * cin * T;
-    for (int i = tid; i < cin * span; i += blockDim.x) {
-        const int ci = i / span, u = i % span;
-        const int t = t0 + u - CNN_HALF;
-        xs[i] = (t >= 0 && t < T) ? xb[(int64_t)ci * T + t] : 0.0f;
-    }
-    __syncthreads();
-    const int tt = (tid % (CONV_TT / CONV_RT)) * CONV_RT;  // first bin of this thread
-    const int cg = tid / (CONV_TT / CONV_RT);               // channel group
-    float acc[CONV_RC][CONV_RT];
-#pragma unroll
-    for (int c = 0; c < CONV_RC; ++c)
-#pragma unroll
-        for (int r = 0; r < CONV_RT; ++r) acc[c][r] = 0.0f;
-    const int co0 = cg * CONV_RC;
-    for (int ci = 0; ci < cin; ++ci) {
-        float xv[CONV_RT + CNN_K - 1];
-#pragma unroll
-        for (int u = 0; u < CONV_RT + CNN_K - 1; ++u) xv[u] = xs[ci * span + tt + u];
-#pragma unroll
-        for (int c = 0; c < CONV_RC; ++c) {
-            if (co0 + c >= cout) break;
-            const float *wr = ws + ((co0 + c) * cin + ci) * CNN_K;
-#pragma unroll
-            for (int k = 0; k < CNN_K; ++k) {
-                const float wk = wr[k];
-#pragma unroll
-                for (int r = 0; r < CONV_RT; ++r) acc[c][r] = fmaf(wk, xv[r + k], acc[c][r]);
-            }
-        }
-    }
-    float *yb = y + (int64_t)b * cout * T;
-#pragma unroll
-    for (int c = 0; c < CONV_RC; ++c) {
-        const int co = co0 + c;
-        if (co >= cout) break;
-        const float bb = bias ? bias[co] : 0.0f;
-#pragma unroll
-        for (int r = 0; r < CONV_RT; ++r) {
-            float v = acc[c][r] + bb;
-            if (relu) v = fmaxf(v, 0.0f);
-            yb[(int64_t)co * T + t0 + tt + r] = v;
-        }
-    }
-}
 
 // ------------------------------------------------------------------------- fused forward pass
 //
@@ -442,108 +376,397 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
                      "n"(NET_TMEM_COLS));
 }
 
-// Weight and bias gradients of one conv layer:
-// dW[co][ci][k] += sum_{b,t} g[b][co][t] x[b][ci][t + k - 4],  db[co] += sum_{b,t} g[b][co][t].
-// One block per (curve, CONV_TT bins): thread (ci, group of 4 co) slides a 9-wide input
-// window along the tile; partial sums are added to the global gradient with atomics.
-__global__ void __launch_bounds__(256)
-cnn_wgrad_kernel(const float *__restrict__ x, const float *__restrict__ g,
-                 float *__restrict__ dw, float *__restrict__ db, int cin, int cout, int T) {
-    extern __shared__ float cs[];
-    const int span = CONV_TT + CNN_K - 1;
-    float *xs = cs;                 // [cin][span]
-    float *gs = cs + cin * span;    // [cout][CONV_TT]
-    const int b = blockIdx.y, t0 = blockIdx.x * CONV_TT, tid = threadIdx.x;
-    const float *xb = x + (int64_t)b * cin * T;
-    const float *gb = g + (int64_t)b * cout * T;
-    for (int i = tid; i < cin * span; i += blockDim.x) {
-        const int ci = i / span, u = i % span;
-        const int t = t0 + u - CNN_HALF;
-        xs[i] = (t >= 0 && t < T) ? xb[(int64_t)ci * T + t] : 0.0f;
-    }
-    for (int i = tid; i < cout * CONV_TT; i += blockDim.x)
-        gs[i] = gb[(int64_t)(i / CONV_TT) * T + t0 + i % CONV_TT];
-    __syncthreads();
-    const int ci = tid % 32, cg = tid / 32;  // 32 input channels x 8 groups of 4 outputs
-    if (ci < cin && cg * 4 < cout) {
-        float acc[4][CNN_K];
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int k = 0; k < CNN_K; ++k) acc[c][k] = 0.0f;
-        float win[CNN_K];
-#pragma unroll
-        for (int k = 0; k < CNN_K; ++k) win[k] = xs[ci * span + k];
-        for (int t = 0; t < CONV_TT; ++t) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int co = cg * 4 + c;
-                const float gv = co < cout ? gs[co * CONV_TT + t] : 0.0f;
-#pragma unroll
-                for (int k = 0; k < CNN_K; ++k) acc[c][k] = fmaf(gv, win[k], acc[c][k]);
-            }
-#pragma unroll
-            for (int k = 0; k < CNN_K - 1; ++k) win[k] = win[k + 1];
-            win[CNN_K - 1] = xs[ci * span + min(t + CNN_K, span - 1)];
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const int co = cg * 4 + c;
-            if (co >= cout) break;
-#pragma unroll
-            for (int k = 0; k < CNN_K; ++k) atomicAdd(&dw[(co * cin + ci) * CNN_K + k], acc[c][k]);
-        }
-    }
-    if (tid < cout) {
-        float s = 0.0f;
-        for (int t = 0; t < CONV_TT; ++t) s += gs[tid * CONV_TT + t];
-        atomicAdd(&db[tid], s);
-    }
-}
-
-// wt[ci][co][k] = w[co][ci][8 - k]: the input gradient is a conv of g with these weights.
-__global__ void cnn_transpose_kernel(const __nv_bfloat16 *__restrict__ w,
-                                     __nv_bfloat16 *__restrict__ wt, int cin, int cout) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cin * cout * CNN_K) return;
-    const int k = i % CNN_K, co = (i / CNN_K) % cout, ci = i / (CNN_K * cout);
-    wt[i] = w[(co * cin + ci) * CNN_K + (CNN_K - 1 - k)];
-}
-
-// g *= (a > 0): back through ReLU.
-__global__ void cnn_relu_back_kernel(float *__restrict__ g, const float *__restrict__ a,
-                                     int64_t n) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        if (!(a[i] > 0.0f)) g[i] = 0.0f;
-}
-
+// ------------------------------------------------------------------------- backward pass
+//
 // Weighted binary cross-entropy with logits, mean over bins:
 // l = w+ y softplus(-z) + (1 - y) softplus(z);  dl/dz = (sigmoid(z) (w+ y + 1 - y) - w+ y) / n.
-__global__ void cnn_bce_kernel(const float *__restrict__ z, const float *__restrict__ y,
-                               float *__restrict__ g, int64_t n, float wpos,
-                               double *__restrict__ loss) {
-    __shared__ double red[32];
-    double acc = 0.0;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const float inv = 1.0f / (float)n;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const float zi = z[i], yi = y[i];
-        const float sp_pos = fmaxf(zi, 0.0f) + log1pf(expf(-fabsf(zi)));  // softplus(z)
-        const float sp_neg = sp_pos - zi;                                 // softplus(-z)
-        acc += (double)(wpos * yi * sp_neg + (1.0f - yi) * sp_pos);
-        const float s = 1.0f / (1.0f + expf(-zi));
-        g[i] = (s * (wpos * yi + 1.0f - yi) - wpos * yi) * inv;
+__device__ __forceinline__ float bce_grad(float z, float y, float wpos, float inv) {
+    const float s = 1.0f / (1.0f + expf(-z));
+    return (s * (wpos * y + 1.0f - y) - wpos * y) * inv;
+}
+__device__ __forceinline__ float bce_loss(float z, float y, float wpos) {
+    const float sp_pos = fmaxf(z, 0.0f) + log1pf(expf(-fabsf(z)));  // softplus(z)
+    return wpos * y * (sp_pos - z) + (1.0f - y) * sp_pos;            // softplus(-z) = sp_pos - z
+}
+
+// Gradients G_l of the pre-activations of layers 2, 1 and 0 (and the loss) for BACK_OUT bins of
+// one curve per tile, in one kernel: the gradient of a layer's input is a conv of its output's
+// gradient with the flipped, transposed weights, so the same tensor-core tiles as the forward
+// pass run in reverse: G_3 (one channel) -> G_2 in FP32, G_2 -> G_1 -> G_0 as matrix
+// instructions, each masked where the layer's activation is not positive (ReLU). Rows: G_2's
+// row i is bin t0 - 8 + i, G_1's row r bin t0 - 4 + r, G_0's row r bin t0 + r.
+// Measured with the weight gradients below (32 curves, 16 durations): 940 us a step when each
+// layer was a transpose, an FP32 conv and a mask kernel and the weight gradients met in atomics.
+constexpr int BACK_OUT = NET_ROWS - 8;
+constexpr int BACK_G4 = NET_XROWS + 8;  // bins of G_3 a tile needs
+inline size_t back_smem() {
+    return (size_t)3 * NET_PART + 2 * net_wbytes(4) + (CNN_C * CNN_K + BACK_G4) * sizeof(float);
+}
+struct back_args {
+    const __nv_bfloat16 *w1, *w2, *w3;       // layers 1, 2, 3: [co][ci][9]
+    const float *logits, *labels;            // [B][T]
+    const float *act1, *act2, *act3;         // outputs of layers 0, 1, 2: [B][32][T]
+    float *g0, *g1, *g2;                     // [B][32][T]
+    double *loss;
+    float wpos;
+    int64_t n;                               // bins of the batch
+};
+
+__global__ void __launch_bounds__(NET_THREADS, 2)
+cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
+    extern __shared__ __align__(128) unsigned char net_raw[];
+    __shared__ uint64_t done[2];
+    __shared__ uint32_t s_tmem;
+    __shared__ double s_loss[NET_THREADS / 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t x0 = smem_u32(net_raw), w0 = x0 + 3 * NET_PART;
+    unsigned char *wraw = net_raw + 3 * NET_PART;
+    float *w3 = reinterpret_cast<float *>(wraw + 2 * net_wbytes(4));  // [ci][9]
+    float *g3 = w3 + CNN_C * CNN_K;                                   // [BACK_G4]
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(&s_tmem)),
+                     "n"(NET_TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) red[wid] = acc;
+    if (tid == 0) {
+        mbar_init(&done[0], 1);
+        mbar_init(&done[1], 1);
+        fence_mbar_init();
+    }
+    // flipped, transposed weights of layers 2 and 1: [tap][unit of co][ci][8 co]
+    for (int l = 0; l < 2; ++l) {
+        const __nv_bfloat16 *w = l == 0 ? ar.w2 : ar.w1;
+        __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(wraw + l * net_wbytes(4));
+        for (int i = tid; i < CNN_K * 4 * CNN_C * 8; i += NET_THREADS) {
+            const int e = i & 7, ci = (i >> 3) & 31, u = (i >> 8) & 3, k = i >> 10;
+            dst[i] = w[((u * 8 + e) * CNN_C + ci) * CNN_K + (CNN_K - 1 - k)];
+        }
+    }
+    for (int i = tid; i < CNN_C * CNN_K; i += NET_THREADS) w3[i] = __bfloat162float(ar.w3[i]);
+    fence_proxy_async();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (wid == 0) {
-        acc = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, o);
-        if (lane == 0) atomicAdd(loss, acc / (double)n);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tm = s_tmem;
+    const float inv = 1.0f / (float)ar.n;
+    double loss = 0.0;
+    uint32_t phase = 0;
+    bool failed = false;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int b = tile / tiles_per_curve;
+        const int t0 = (tile - b * tiles_per_curve) * BACK_OUT;
+        const int own_end = min(T, t0 + BACK_OUT);
+        for (int i = tid; i < BACK_G4; i += NET_THREADS) {  // G_3 and the loss, bin t0 - 12 + i
+            const int t = t0 - 12 + i;
+            float g = 0.0f;
+            if (t >= 0 && t < T) {
+                const float z = ar.logits[(int64_t)b * T + t], y = ar.labels[(int64_t)b * T + t];
+                g = bce_grad(z, y, ar.wpos, inv);
+                if (t >= t0 && t < own_end) loss += (double)bce_loss(z, y, ar.wpos);
+            }
+            g3[i] = g;
+        }
+        __syncthreads();
+        for (int it = tid; it < NET_XROWS * 4; it += NET_THREADS) {
+            const int u = it / NET_XROWS, i = it - u * NET_XROWS;
+            const int t = t0 - 8 + i;
+            const bool inside = t >= 0 && t < T;
+            const int64_t at = ((int64_t)b * CNN_C + u * 8) * T + t;
+            float a[8], v[8], g[CNN_K];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) a[e] = inside ? ar.act3[at + (int64_t)e * T] : 0.0f;
+#pragma unroll
+            for (int k = 0; k < CNN_K; ++k) g[k] = g3[i + 8 - k];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float sum = 0.0f;
+#pragma unroll
+                for (int k = 0; k < CNN_K; ++k)
+                    sum = fmaf(g[k], w3[(u * 8 + e) * CNN_K + k], sum);
+                v[e] = a[e] > 0.0f ? sum : 0.0f;
+                if (inside && t >= t0 && t < own_end) ar.g2[at + (int64_t)e * T] = v[e];
+            }
+            net_store_row(x0 + (uint32_t)(u * NET_UNIT + i * 16), v);
+        }
+        fence_proxy_async();
+        __syncthreads();
+        for (int l = 0; l < 2; ++l) {
+            if (tid == 0) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (int mb = 0; mb < 2; ++mb) {
+                    net_layer_mma<4>(tm + (uint32_t)(mb * NET_GRP * CNN_C),
+                                     net_desc_lo(x0 + (uint32_t)(mb * 128 * 16), NET_UNIT),
+                                     net_desc_lo(w0 + (uint32_t)(l * net_wbytes(4)), CNN_C * 16));
+                    net_commit(&done[mb]);
+                }
+            }
+            __syncwarp();
+            const int mb = warp >> 2, r = mb * 128 + (warp & 3) * 32 + lane;
+            const int t = t0 - 4 + 4 * l + r;
+            const bool inside = t >= 0 && t < T;
+            const bool own = inside && t >= t0 && t < own_end;
+            const int64_t at = (int64_t)b * CNN_C * T + t;
+            const float *act = l == 0 ? ar.act2 : ar.act1;
+            float *out = l == 0 ? ar.g1 : ar.g0;
+            uint32_t mask = 0u;  // channels whose activation is positive, read under the instructions
+            if (inside)
+#pragma unroll
+                for (int c = 0; c < CNN_C; ++c)
+                    mask |= (act[at + (int64_t)c * T] > 0.0f ? 1u : 0u) << c;
+            const bool ok = mbar_wait(&done[mb], phase);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float v[16], o[16];
+                net_tmem_load(v, src + h * 16);
+                net_tmem_wait(v);
+#pragma unroll
+                for (int g = 1; g < NET_GRP; ++g) {
+                    net_tmem_load(o, src + g * CNN_C + h * 16);
+                    net_tmem_wait(o);
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) v[c] += o[c];
+                }
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    v[c] = (mask >> (h * 16 + c)) & 1u ? v[c] : 0.0f;
+                    if (own) out[at + (int64_t)(h * 16 + c) * T] = v[c];
+                }
+                if (l == 0) {
+                    net_store_row(x0 + (uint32_t)(2 * h * NET_UNIT + r * 16), v);
+                    net_store_row(x0 + (uint32_t)((2 * h + 1) * NET_UNIT + r * 16), v + 8);
+                }
+            }
+            phase ^= 1u;
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            fence_proxy_async();
+            failed = __syncthreads_or(!ok);
+            if (failed) break;
+        }
+        if (failed) {  // a wait gave up: the loss says so
+            mbar_wait(&done[0], phase ^ 1u);  // (bounded) before the tensor memory goes
+            mbar_wait(&done[1], phase ^ 1u);
+            loss = __longlong_as_double(0x7ff8000000000000ll);
+            break;
+        }
     }
+    for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xFFFFFFFFu, loss, o);
+    if (lane == 0) s_loss[warp] = loss;
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (tid == 0) {
+        for (int x = 1; x < NET_THREADS / 32; ++x) loss += s_loss[x];
+        atomicAdd(ar.loss, loss / (double)ar.n);
+    }
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm),
+                     "n"(NET_TMEM_COLS));
+}
+
+// Weight and bias gradients of every layer in one launch:
+// dW[co][ci][k] = sum_{b,t} G[b][co][t] x[b][ci][t + k - 4],  db[co] = sum_{b,t} G[b][co][t].
+// Each layer has its share of the blocks; a block goes through its tiles of bins with the sums in
+// registers and leaves one partial gradient, which cnn_grad_sum_kernel adds over the blocks (no
+// atomics: 4.7 M scattered ones per layer were most of the time of the kernel this replaces,
+// 150 us for a 32 -> 32 layer of 32 curves). Thread: one input channel x 8 output channels x 9
+// taps over WG_SUB bins of the tile: 36 packed FP32x2 multiply-adds per bin on the pair (G of two
+// output channels) x (x, x), so the FMA pipe is the bound; the 9-wide input window rotates
+// through registers, G comes as broadcast 16-byte loads.
+constexpr int WG_THREADS = 256;
+constexpr int WG_SUB = 63;   // bins per thread and tile (a multiple of the taps: the window's rotation)
+constexpr int WG_LDG = 36;   // floats per bin of the staged G (16-byte aligned, few bank conflicts)
+constexpr int WG_LAST = 128; // bins per tile of the last layer
+struct wgrad_job {
+    const float *x, *g;  // input [B][cin][T], gradient [B][32][T] (last layer: from the logits)
+    float *part;         // [blocks][size] partial gradients: W then b
+    int cin, cout, first, blocks, size;
+};
+struct wgrad_args {
+    wgrad_job job[CNN_LAYERS];
+    const float *logits, *labels;  // [B][T]
+    float wpos;
+    int64_t n;
+    int B, T;
+};
+// Input channels as lanes hold them (16 or 32), thread groups along the bins, bins per tile.
+__host__ __device__ constexpr int wg_cinp(int cin) { return cin <= 16 ? 16 : 32; }
+__host__ __device__ constexpr int wg_subs(int cin) { return WG_THREADS / 4 / wg_cinp(cin); }
+__host__ __device__ constexpr int wg_tile(int cin) { return wg_subs(cin) * WG_SUB; }
+constexpr size_t WG_SMEM = (16 * (4 * WG_SUB + 9) + 4 * WG_SUB * WG_LDG) * sizeof(float);
+static_assert(WG_SMEM >= (32 * (2 * WG_SUB + 9) + 2 * WG_SUB * WG_LDG) * sizeof(float) &&
+                  WG_SMEM >= 72 * 128 * sizeof(float) &&
+                  WG_SMEM >= (CNN_C * (WG_LAST + 9) + WG_LAST) * sizeof(float),
+              "weight gradient staging");
+
+__device__ void wgrad_last(const wgrad_args &ar, const wgrad_job &jb, float *smem) {
+    constexpr int XS = WG_LAST + 9;
+    float *xs = smem, *gs = smem + CNN_C * XS;
+    const int tid = threadIdx.x, ci = tid & 31, warp = tid >> 5;
+    const int T = ar.T, per = (T + WG_LAST - 1) / WG_LAST;
+    const float inv = 1.0f / (float)ar.n;
+    float acc[CNN_K], db = 0.0f;
+#pragma unroll
+    for (int k = 0; k < CNN_K; ++k) acc[k] = 0.0f;
+    for (int tile = blockIdx.x - jb.first; tile < per * ar.B; tile += jb.blocks) {
+        const int b = tile / per, t0 = (tile - b * per) * WG_LAST;
+        __syncthreads();
+        for (int i = tid; i < CNN_C * (WG_LAST + 8); i += WG_THREADS) {
+            const int c = i / (WG_LAST + 8), u = i - c * (WG_LAST + 8), t = t0 - 4 + u;
+            xs[c * XS + u] = t >= 0 && t < T ? jb.x[((int64_t)b * CNN_C + c) * T + t] : 0.0f;
+        }
+        for (int u = tid; u < WG_LAST; u += WG_THREADS) {
+            const int64_t at = (int64_t)b * T + t0 + u;
+            gs[u] = t0 + u < T ? bce_grad(ar.logits[at], ar.labels[at], ar.wpos, inv) : 0.0f;
+        }
+        __syncthreads();
+        const int u0 = warp * (WG_LAST / 8);
+        for (int u = u0; u < u0 + WG_LAST / 8; ++u) {
+            const float g = gs[u];
+            db += g;
+#pragma unroll
+            for (int k = 0; k < CNN_K; ++k) acc[k] = fmaf(g, xs[ci * XS + u + k], acc[k]);
+        }
+    }
+    __syncthreads();
+    float *red = smem;  // [8 warps][32][9], then [8] biases
+#pragma unroll
+    for (int k = 0; k < CNN_K; ++k) red[(warp * CNN_C + ci) * CNN_K + k] = acc[k];
+    if (ci == 0) red[8 * CNN_C * CNN_K + warp] = db;
+    __syncthreads();
+    float *out = jb.part + (int64_t)(blockIdx.x - jb.first) * jb.size;
+    for (int i = tid; i < CNN_C * CNN_K; i += WG_THREADS) {
+        float v = 0.0f;
+        for (int w = 0; w < 8; ++w) v += red[w * CNN_C * CNN_K + i];
+        out[i] = v;
+    }
+    if (tid == 0) {
+        float v = 0.0f;
+        for (int w = 0; w < 8; ++w) v += red[8 * CNN_C * CNN_K + w];
+        out[CNN_C * CNN_K] = v;
+    }
+}
+
+__global__ void __launch_bounds__(WG_THREADS, 2) cnn_wgrad_kernel(wgrad_args ar) {
+    extern __shared__ __align__(16) float wg_smem[];
+    int l = 0;
+    while (l < CNN_LAYERS - 1 && (int)blockIdx.x >= ar.job[l].first + ar.job[l].blocks) ++l;
+    const wgrad_job jb = ar.job[l];
+    if (l == CNN_LAYERS - 1) {  // uniform over the block
+        wgrad_last(ar, jb, wg_smem);
+        return;
+    }
+    const int tid = threadIdx.x, cin = jb.cin, T = ar.T;
+    const int cinp = wg_cinp(cin), subs = wg_subs(cin), tile_n = wg_tile(cin), XS = tile_n + 9;
+    float *xs = wg_smem, *gs = wg_smem + ((cinp * XS + 3) & ~3);
+    const int ci = tid % cinp, rest = tid / cinp, cg = rest & 3, sub = rest >> 2;
+    const int per = (T + tile_n - 1) / tile_n;
+    unsigned long long acc[4][CNN_K];  // (output channels 2 p, 2 p + 1 of the thread's eight)
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int k = 0; k < CNN_K; ++k) acc[p][k] = 0ull;
+    float db = 0.0f;
+    for (int tile = blockIdx.x - jb.first; tile < per * ar.B; tile += jb.blocks) {
+        const int b = tile / per, t0 = (tile - b * per) * tile_n;
+        __syncthreads();  // the previous tile is read
+        const float *xb = jb.x + (int64_t)b * cin * T, *gb = jb.g + (int64_t)b * CNN_C * T;
+        for (int c = tid >> 5; c < cinp; c += WG_THREADS / 32)
+            for (int u = tid & 31; u < tile_n + 8; u += 32) {
+                const int t = t0 - 4 + u;
+                xs[c * XS + u] = c < cin && t >= 0 && t < T ? xb[(int64_t)c * T + t] : 0.0f;
+            }
+        for (int c = tid >> 5; c < CNN_C; c += WG_THREADS / 32)
+            for (int u = tid & 31; u < tile_n; u += 32)
+                gs[u * WG_LDG + c] = t0 + u < T ? gb[(int64_t)c * T + t0 + u] : 0.0f;
+        __syncthreads();
+        const float *xr = xs + ci * XS + sub * WG_SUB, *gr = gs + sub * WG_SUB * WG_LDG + cg * 8;
+        unsigned long long win[CNN_K];
+#pragma unroll
+        for (int k = 0; k < CNN_K; ++k) win[k] = pack2(make_float2(xr[k], xr[k]));
+        for (int it = 0; it < WG_SUB; it += CNN_K)
+#pragma unroll
+            for (int s = 0; s < CNN_K; ++s) {
+                const ulonglong2 ga = *reinterpret_cast<const ulonglong2 *>(gr + (it + s) * WG_LDG);
+                const ulonglong2 gc =
+                    *reinterpret_cast<const ulonglong2 *>(gr + (it + s) * WG_LDG + 4);
+                const unsigned long long g[4] = {ga.x, ga.y, gc.x, gc.y};
+                const float xn = xr[it + s + CNN_K];
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int k = 0; k < CNN_K; ++k)
+                        asm("fma.rn.f32x2 %0, %1, %2, %0;"
+                            : "+l"(acc[p][k])
+                            : "l"(g[p]), "l"(win[(s + k) % CNN_K]));
+                win[s] = pack2(make_float2(xn, xn));
+            }
+        for (int u = tid >> 5; u < tile_n; u += WG_THREADS / 32) db += gs[u * WG_LDG + (tid & 31)];
+    }
+    // the thread groups' sums of each weight, then this block's partial gradient
+    float *red = wg_smem;  // [72][128]
+    const int slot = cg * cinp + ci;
+    for (int x = 1; x < subs; ++x) {
+        __syncthreads();
+        if (sub == x)
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int k = 0; k < CNN_K; ++k) {
+                    const float2 v = unpack2(acc[p][k]);
+                    red[((p * CNN_K + k) * 2) * 128 + slot] = v.x;
+                    red[((p * CNN_K + k) * 2 + 1) * 128 + slot] = v.y;
+                }
+        __syncthreads();
+        if (sub == 0)
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int k = 0; k < CNN_K; ++k) {
+                    float2 v = unpack2(acc[p][k]);
+                    v.x += red[((p * CNN_K + k) * 2) * 128 + slot];
+                    v.y += red[((p * CNN_K + k) * 2 + 1) * 128 + slot];
+                    acc[p][k] = pack2(v);
+                }
+    }
+    float *out = jb.part + (int64_t)(blockIdx.x - jb.first) * jb.size;
+    if (sub == 0 && ci < cin)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int k = 0; k < CNN_K; ++k) {
+                const float2 v = unpack2(acc[p][k]);
+                const int co = cg * 8 + 2 * p;
+                out[(co * cin + ci) * CNN_K + k] = v.x;
+                out[((co + 1) * cin + ci) * CNN_K + k] = v.y;
+            }
+    __syncthreads();
+    red[tid] = db;
+    __syncthreads();
+    if (tid < CNN_C) {
+        float v = 0.0f;
+        for (int w = 0; w < WG_THREADS / 32; ++w) v += red[w * 32 + tid];
+        out[CNN_C * cin * CNN_K + tid] = v;
+    }
+}
+
+// The gradient: the blocks' partial gradients of each layer added in block order.
+__global__ void cnn_grad_sum_kernel(wgrad_args ar, float *__restrict__ grads) {
+    const wgrad_job jb = ar.job[blockIdx.y];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= jb.size) return;
+    float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    int x = 0;
+    for (; x + 4 <= jb.blocks; x += 4)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] += jb.part[(int64_t)(x + k) * jb.size + i];
+    for (; x < jb.blocks; ++x) v[0] += jb.part[(int64_t)x * jb.size + i];
+    int64_t off = 0;
+    for (int l = 0; l < (int)blockIdx.y; ++l) off += ar.job[l].size;
+    grads[off + i] = (v[0] + v[1]) + (v[2] + v[3]);
 }
 
 __global__ void cnn_round_kernel(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wb,
@@ -780,9 +1003,10 @@ struct cetra_cnn {
     int ch_in[CNN_LAYERS], ch_out[CNN_LAYERS];
     int64_t w_off[CNN_LAYERS], b_off[CNN_LAYERS], n_params = 0;
     float *d_params = nullptr, *d_grads = nullptr, *d_m = nullptr, *d_v = nullptr;
-    __nv_bfloat16 *d_wb = nullptr, *d_wt = nullptr;  // BF16 weights, transposed scratch
+    __nv_bfloat16 *d_wb = nullptr;  // BF16 weights
     float *d_act[CNN_LAYERS + 1] = {};  // act[0] = log1p(features), act[l + 1] = layer l output
-    float *d_g = nullptr, *d_g2 = nullptr;  // gradient buffers [max_batch][32][T]
+    float *d_g[CNN_LAYERS - 1] = {};  // gradients of layers 0 .. 2 [max_batch][32][T]
+    float *d_part = nullptr;          // partial weight gradients of the blocks
     double *d_loss = nullptr;
     void *d_mem = nullptr;
     int adam_step = 0;
@@ -794,21 +1018,9 @@ int cnn_fail(cetra_ctx *ctx, cudaError_t e, const char *what) {
     return set_error(ctx, CETRA_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
-size_t conv_smem(int cin, int cout) {
-    return ((size_t)cout * cin * CNN_K + (size_t)cin * (CONV_TT + CNN_K - 1)) * sizeof(float);
-}
-size_t wgrad_smem(int cin, int cout) {
-    return ((size_t)cin * (CONV_TT + CNN_K - 1) + (size_t)cout * CONV_TT) * sizeof(float);
-}
-
-cudaError_t conv(cetra_ctx *ctx, const float *x, const __nv_bfloat16 *w, const float *bias,
-                 float *y, int cin, int cout, int T, int B, int relu) {
-    dim3 grid((unsigned)(T / CONV_TT), (unsigned)B);
-    cnn_conv_kernel<<<grid, CONV_THREADS, conv_smem(cin, cout), ctx->stream>>>(x, w, bias, y, cin,
-                                                                             cout, T, relu);
-    ctx->launches++;
-    return cudaGetLastError();
-}
+// Blocks of the weight-gradient launch (two per SM), and the largest partial gradient.
+int wgrad_blocks(int num_sms) { return 2 * num_sms; }
+constexpr size_t WG_PART = (size_t)CNN_C * CNN_C * CNN_K + CNN_C;
 
 // The forward pass: probabilities of B curves into prob, or (prob NULL, training) the layers'
 // activations and the logits into the network's buffers.
@@ -845,7 +1057,7 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
                      cetra_cnn **out) {
     if (!ctx || !out) return set_error(ctx, CETRA_EINVAL, "cnn_create: NULL argument");
     *out = nullptr;
-    if (in_channels < 1 || in_channels > CNN_C || n_bins < CONV_TT || n_bins % CONV_TT ||
+    if (in_channels < 1 || in_channels > CNN_C || n_bins < 256 || n_bins % 256 ||
         max_batch < 1)
         return set_error(ctx, CETRA_EINVAL,
                          "cnn_create: need 1 <= in_channels <= 32, n_bins a multiple of 256, max_batch >= 1");
@@ -876,8 +1088,10 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
     }
     const size_t P = (size_t)off;
     const size_t act = (size_t)max_batch * CNN_C * n_bins;
-    const size_t bytes = P * sizeof(float) * 4 + P * sizeof(__nv_bfloat16) * 2 + 256 * 8 +
-                         act * sizeof(float) * (CNN_LAYERS + 1 + 2) + 1024;
+    const size_t logits = (size_t)max_batch * n_bins;
+    const size_t part = (size_t)wgrad_blocks(ctx->num_sms) * WG_PART;
+    const size_t bytes = P * sizeof(float) * 4 + P * sizeof(__nv_bfloat16) + 256 * 16 +
+                         (act * (CNN_LAYERS + CNN_LAYERS - 1) + logits + part) * sizeof(float);
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
     if (!e) e = cudaMalloc(&n->d_mem, bytes);
@@ -896,11 +1110,11 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
     n->d_m = reinterpret_cast<float *>(take(P * 4));
     n->d_v = reinterpret_cast<float *>(take(P * 4));
     n->d_wb = reinterpret_cast<__nv_bfloat16 *>(take(P * 2));
-    n->d_wt = reinterpret_cast<__nv_bfloat16 *>(take(P * 2));
     n->d_loss = reinterpret_cast<double *>(take(8));
-    for (int l = 0; l <= CNN_LAYERS; ++l) n->d_act[l] = reinterpret_cast<float *>(take(act * 4));
-    n->d_g = reinterpret_cast<float *>(take(act * 4));
-    n->d_g2 = reinterpret_cast<float *>(take(act * 4));
+    for (int l = 0; l < CNN_LAYERS; ++l) n->d_act[l] = reinterpret_cast<float *>(take(act * 4));
+    n->d_act[CNN_LAYERS] = reinterpret_cast<float *>(take(logits * 4));
+    for (float *&g : n->d_g) g = reinterpret_cast<float *>(take(act * 4));
+    n->d_part = reinterpret_cast<float *>(take(part * 4));
     e = cudaMemcpy(n->d_params, init.data(), P * 4, cudaMemcpyHostToDevice);
     if (!e) e = cudaMemset(n->d_m, 0, P * 4);
     if (!e) e = cudaMemset(n->d_v, 0, P * 4);
@@ -909,11 +1123,11 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
             e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)net_smem(CNN_C));
     if (!e)
-        e = cudaFuncSetAttribute(cnn_conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)conv_smem(CNN_C, CNN_C));
+        e = cudaFuncSetAttribute(cnn_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)back_smem());
     if (!e)
         e = cudaFuncSetAttribute(cnn_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)wgrad_smem(CNN_C, CNN_C));
+                                 (int)WG_SMEM);
     if (!e) e = round_weights(ctx, n);
     if (!e) e = cudaStreamSynchronize(ctx->stream);
     if (e) {
@@ -986,38 +1200,76 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
     if (!e) e = forward(ctx, n, d_features, B, nullptr);
-    if (!e) e = cudaMemsetAsync(n->d_grads, 0, (size_t)n->n_params * 4, ctx->stream);
     if (!e) e = cudaMemsetAsync(n->d_loss, 0, sizeof(double), ctx->stream);
-    const int64_t m = (int64_t)B * T;
     if (!e) {
-        cnn_bce_kernel<<<grid_for(m, 256, ctx->num_sms), 256, 0, ctx->stream>>>(
-            n->d_act[CNN_LAYERS], d_labels, n->d_g, m, pos_weight, n->d_loss);
-        ctx->launches++;
-        e = cudaGetLastError();
-    }
-    float *g = n->d_g, *g_next = n->d_g2;
-    for (int l = CNN_LAYERS - 1; l >= 0 && !e; --l) {
-        const int cin = n->ch_in[l], cout = n->ch_out[l];
-        if (l < CNN_LAYERS - 1) {  // back through this layer's ReLU
-            const int64_t cnt = (int64_t)B * cout * T;
-            cnn_relu_back_kernel<<<grid_for(cnt, 256, ctx->num_sms), 256, 0, ctx->stream>>>(
-                g, n->d_act[l + 1], cnt);
+        back_args ar{};
+        ar.w1 = n->d_wb + n->w_off[1];
+        ar.w2 = n->d_wb + n->w_off[2];
+        ar.w3 = n->d_wb + n->w_off[3];
+        ar.logits = n->d_act[CNN_LAYERS];
+        ar.labels = d_labels;
+        ar.act1 = n->d_act[1];
+        ar.act2 = n->d_act[2];
+        ar.act3 = n->d_act[3];
+        ar.g0 = n->d_g[0];
+        ar.g1 = n->d_g[1];
+        ar.g2 = n->d_g[2];
+        ar.loss = n->d_loss;
+        ar.wpos = pos_weight;
+        ar.n = (int64_t)B * T;
+        const int per = (T + BACK_OUT - 1) / BACK_OUT;
+        if ((int64_t)per * B > 2147483647) e = cudaErrorInvalidConfiguration;
+        const unsigned blocks =
+            (unsigned)std::min<int64_t>((int64_t)per * B, 2 * (int64_t)ctx->num_sms);
+        if (!e) {
+            cnn_back_kernel<<<blocks, NET_THREADS, back_smem(), ctx->stream>>>(ar, T, per * B, per);
             ctx->launches++;
-            if ((e = cudaGetLastError())) break;
+            e = cudaGetLastError();
         }
-        dim3 grid((unsigned)(T / CONV_TT), (unsigned)B);
-        cnn_wgrad_kernel<<<grid, 256, wgrad_smem(cin, cout), ctx->stream>>>(
-            n->d_act[l], g, n->d_grads + n->w_off[l], n->d_grads + n->b_off[l], cin, cout, T);
-        ctx->launches++;
-        if ((e = cudaGetLastError())) break;
-        if (l > 0) {  // gradient of the layer input: conv of g with the flipped, transposed weights
-            const int nw = cin * cout * CNN_K;
-            cnn_transpose_kernel<<<(nw + 255) / 256, 256, 0, ctx->stream>>>(
-                n->d_wb + n->w_off[l], n->d_wt, cin, cout);
+    }
+    if (!e) {
+        // every layer's share of the blocks by its multiply-adds (the last layer is bound by
+        // reading its input: as a 32 -> 8 layer)
+        wgrad_args ar{};
+        ar.logits = n->d_act[CNN_LAYERS];
+        ar.labels = d_labels;
+        ar.wpos = pos_weight;
+        ar.n = (int64_t)B * T;
+        ar.B = B;
+        ar.T = T;
+        const int slots = wgrad_blocks(ctx->num_sms);
+        double weight[CNN_LAYERS], total = 0.0;
+        for (int l = 0; l < CNN_LAYERS; ++l)
+            total += weight[l] = l == CNN_LAYERS - 1 ? 8.0 : wg_cinp(n->ch_in[l]);
+        int first = 0;
+        float *part = n->d_part;
+        for (int l = 0; l < CNN_LAYERS; ++l) {
+            wgrad_job &jb = ar.job[l];
+            jb.x = n->d_act[l];
+            jb.g = l < CNN_LAYERS - 1 ? n->d_g[l] : nullptr;
+            jb.cin = n->ch_in[l];
+            jb.cout = n->ch_out[l];
+            jb.size = jb.cout * jb.cin * CNN_K + jb.cout;
+            const int tile = l < CNN_LAYERS - 1 ? wg_tile(jb.cin) : WG_LAST;
+            const int64_t tiles = (int64_t)((T + tile - 1) / tile) * B;
+            if (tiles > 2147483647) e = cudaErrorInvalidConfiguration;
+            jb.first = first;
+            jb.blocks = (int)std::max<int64_t>(
+                1, std::min<int64_t>(tiles, (int64_t)(slots * weight[l] / total)));
+            jb.part = part;
+            part += (size_t)jb.blocks * jb.size;
+            first += jb.blocks;
+        }
+        if (!e) {
+            cnn_wgrad_kernel<<<first, WG_THREADS, WG_SMEM, ctx->stream>>>(ar);
             ctx->launches++;
-            if ((e = cudaGetLastError())) break;
-            if ((e = conv(ctx, g, n->d_wt, nullptr, g_next, cout, cin, T, B, 0))) break;
-            std::swap(g, g_next);
+            e = cudaGetLastError();
+        }
+        if (!e) {
+            dim3 grid((unsigned)((WG_PART + 127) / 128), CNN_LAYERS);
+            cnn_grad_sum_kernel<<<grid, 128, 0, ctx->stream>>>(ar, n->d_grads);
+            ctx->launches++;
+            e = cudaGetLastError();
         }
     }
     if (!e && loss) e = cudaMemcpyAsync(loss, n->d_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
