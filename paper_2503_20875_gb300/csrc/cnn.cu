@@ -574,8 +574,10 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
 // atomics: 4.7 M scattered ones per layer were most of the time of the kernel this replaces,
 // 150 us for a 32 -> 32 layer of 32 curves). Thread: one input channel x 8 output channels x 9
 // taps over WG_SUB bins of the tile: 36 packed FP32x2 multiply-adds per bin on the pair (G of two
-// output channels) x (x, x), so the FMA pipe is the bound; the 9-wide input window rotates
-// through registers, G comes as broadcast 16-byte loads.
+// output channels) x (x, x), so the FMA pipe is the bound (55 % busy, 153 us for 32 curves); the
+// 9-wide input window rotates through registers, G comes as broadcast 16-byte loads. Tiles are
+// staged by asynchronous copies, the next one under the arithmetic of this one, and handed out as
+// blocks come free (206 us with plain loads and a fixed share).
 constexpr int WG_THREADS = 256;
 constexpr int WG_SUB = 63;   // bins per thread and tile (a multiple of the taps: the window's rotation)
 constexpr int WG_LDG = 36;   // floats per bin of the staged G (16-byte aligned, few bank conflicts)
@@ -588,6 +590,7 @@ struct wgrad_job {
 struct wgrad_args {
     wgrad_job job[CNN_LAYERS];
     const float *logits, *labels;  // [B][T]
+    int *next;                     // [layer] tiles handed out beyond each block's first (zeroed)
     float wpos;
     int64_t n;
     int B, T;
@@ -596,11 +599,38 @@ struct wgrad_args {
 __host__ __device__ constexpr int wg_cinp(int cin) { return cin <= 16 ? 16 : 32; }
 __host__ __device__ constexpr int wg_subs(int cin) { return WG_THREADS / 4 / wg_cinp(cin); }
 __host__ __device__ constexpr int wg_tile(int cin) { return wg_subs(cin) * WG_SUB; }
-constexpr size_t WG_SMEM = (16 * (4 * WG_SUB + 9) + 4 * WG_SUB * WG_LDG) * sizeof(float);
-static_assert(WG_SMEM >= (32 * (2 * WG_SUB + 9) + 2 * WG_SUB * WG_LDG) * sizeof(float) &&
-                  WG_SMEM >= 72 * 128 * sizeof(float) &&
-                  WG_SMEM >= (CNN_C * (WG_LAST + 9) + WG_LAST) * sizeof(float),
+constexpr int WG_STAGE = 16 * (4 * WG_SUB + 9) + 4 * WG_SUB * WG_LDG;  // floats of a staged tile
+constexpr size_t WG_SMEM = (size_t)2 * WG_STAGE * sizeof(float);
+static_assert(WG_STAGE >= 32 * (2 * WG_SUB + 9) + 2 * WG_SUB * WG_LDG && WG_STAGE % 4 == 0 &&
+                  2 * WG_STAGE >= 72 * 128 && 2 * WG_STAGE >= CNN_C * (WG_LAST + 9) + WG_LAST,
               "weight gradient staging");
+
+// Asynchronous copy of one float (zero when !ok: nothing is read then).
+__device__ __forceinline__ void copy_float(float *dst, const float *src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src),
+                 "r"(ok ? 4 : 0)
+                 : "memory");
+}
+
+// Stage one tile of a layer's input and output gradient (asynchronous; one commit group).
+__device__ __forceinline__ void wgrad_stage(const wgrad_job &jb, int tile, int per, int tile_n,
+                                            int cinp, int T, float *xs, float *gs) {
+    const int b = tile / per, t0 = (tile - b * per) * tile_n, XS = tile_n + 9;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float *xb = jb.x + (int64_t)b * jb.cin * T, *gb = jb.g + (int64_t)b * CNN_C * T;
+    for (int c = warp; c < cinp; c += WG_THREADS / 32)
+        for (int u = lane; u < tile_n + 8; u += 32) {
+            const int t = t0 - 4 + u;
+            const bool ok = c < jb.cin && t >= 0 && t < T;
+            copy_float(&xs[c * XS + u], ok ? xb + (int64_t)c * T + t : jb.x, ok);
+        }
+    for (int c = warp; c < CNN_C; c += WG_THREADS / 32)
+        for (int u = lane; u < tile_n; u += 32) {
+            const bool ok = t0 + u < T;
+            copy_float(&gs[u * WG_LDG + c], ok ? gb + (int64_t)c * T + t0 + u : jb.g, ok);
+        }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
 
 __device__ void wgrad_last(const wgrad_args &ar, const wgrad_job &jb, float *smem) {
     constexpr int XS = WG_LAST + 9;
@@ -614,14 +644,19 @@ __device__ void wgrad_last(const wgrad_args &ar, const wgrad_job &jb, float *sme
     for (int tile = blockIdx.x - jb.first; tile < per * ar.B; tile += jb.blocks) {
         const int b = tile / per, t0 = (tile - b * per) * WG_LAST;
         __syncthreads();
-        for (int i = tid; i < CNN_C * (WG_LAST + 8); i += WG_THREADS) {
-            const int c = i / (WG_LAST + 8), u = i - c * (WG_LAST + 8), t = t0 - 4 + u;
-            xs[c * XS + u] = t >= 0 && t < T ? jb.x[((int64_t)b * CNN_C + c) * T + t] : 0.0f;
-        }
+        for (int c = warp; c < CNN_C; c += WG_THREADS / 32)  // (in flight together)
+            for (int u = ci; u < WG_LAST + 8; u += 32) {
+                const int t = t0 - 4 + u;
+                const bool ok = t >= 0 && t < T;
+                copy_float(&xs[c * XS + u], ok ? jb.x + ((int64_t)b * CNN_C + c) * T + t : jb.x,
+                           ok);
+            }
+        asm volatile("cp.async.commit_group;" ::: "memory");
         for (int u = tid; u < WG_LAST; u += WG_THREADS) {
             const int64_t at = (int64_t)b * T + t0 + u;
             gs[u] = t0 + u < T ? bce_grad(ar.logits[at], ar.labels[at], ar.wpos, inv) : 0.0f;
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
         const int u0 = warp * (WG_LAST / 8);
         for (int u = u0; u < u0 + WG_LAST / 8; ++u) {
@@ -661,7 +696,7 @@ __global__ void __launch_bounds__(WG_THREADS, 2) cnn_wgrad_kernel(wgrad_args ar)
     }
     const int tid = threadIdx.x, cin = jb.cin, T = ar.T;
     const int cinp = wg_cinp(cin), subs = wg_subs(cin), tile_n = wg_tile(cin), XS = tile_n + 9;
-    float *xs = wg_smem, *gs = wg_smem + ((cinp * XS + 3) & ~3);
+    const int g_at = (cinp * XS + 3) & ~3;  // G after the input, in each of the two stages
     const int ci = tid % cinp, rest = tid / cinp, cg = rest & 3, sub = rest >> 2;
     const int per = (T + tile_n - 1) / tile_n;
     unsigned long long acc[4][CNN_K];  // (output channels 2 p, 2 p + 1 of the thread's eight)
@@ -670,19 +705,27 @@ __global__ void __launch_bounds__(WG_THREADS, 2) cnn_wgrad_kernel(wgrad_args ar)
 #pragma unroll
         for (int k = 0; k < CNN_K; ++k) acc[p][k] = 0ull;
     float db = 0.0f;
-    for (int tile = blockIdx.x - jb.first; tile < per * ar.B; tile += jb.blocks) {
-        const int b = tile / per, t0 = (tile - b * per) * tile_n;
-        __syncthreads();  // the previous tile is read
-        const float *xb = jb.x + (int64_t)b * cin * T, *gb = jb.g + (int64_t)b * CNN_C * T;
-        for (int c = tid >> 5; c < cinp; c += WG_THREADS / 32)
-            for (int u = tid & 31; u < tile_n + 8; u += 32) {
-                const int t = t0 - 4 + u;
-                xs[c * XS + u] = c < cin && t >= 0 && t < T ? xb[(int64_t)c * T + t] : 0.0f;
-            }
-        for (int c = tid >> 5; c < CNN_C; c += WG_THREADS / 32)
-            for (int u = tid & 31; u < tile_n; u += 32)
-                gs[u * WG_LDG + c] = t0 + u < T ? gb[(int64_t)c * T + t0 + u] : 0.0f;
+    // tiles after a block's first are handed out as blocks come free: an SM may hold blocks of
+    // layers of different length
+    __shared__ int s_next;
+    const int n_tiles = per * ar.B;
+    int tile = blockIdx.x - jb.first, stage = 0;
+    if (tid == 0) s_next = jb.blocks + atomicAdd(&ar.next[l], 1);
+    if (tile < n_tiles) wgrad_stage(jb, tile, per, tile_n, cinp, T, wg_smem, wg_smem + g_at);
+    __syncthreads();
+    for (int after; tile < n_tiles; tile = after, stage ^= 1) {
+        // the next tile lands in the other stage while this one is used
+        float *xs = wg_smem + stage * WG_STAGE, *gs = xs + g_at;
+        float *xn_s = wg_smem + (stage ^ 1) * WG_STAGE;
+        after = s_next;
+        if (after < n_tiles) {
+            wgrad_stage(jb, after, per, tile_n, cinp, T, xn_s, xn_s + g_at);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
         __syncthreads();
+        if (tid == 0 && after < n_tiles) s_next = jb.blocks + atomicAdd(&ar.next[l], 1);
         const float *xr = xs + ci * XS + sub * WG_SUB, *gr = gs + sub * WG_SUB * WG_LDG + cg * 8;
         unsigned long long win[CNN_K];
 #pragma unroll
@@ -705,6 +748,7 @@ __global__ void __launch_bounds__(WG_THREADS, 2) cnn_wgrad_kernel(wgrad_args ar)
                 win[s] = pack2(make_float2(xn, xn));
             }
         for (int u = tid >> 5; u < tile_n; u += WG_THREADS / 32) db += gs[u * WG_LDG + (tid & 31)];
+        __syncthreads();  // the stage is read before the next copies into it
     }
     // the thread groups' sums of each weight, then this block's partial gradient
     float *red = wg_smem;  // [72][128]
@@ -753,20 +797,33 @@ __global__ void __launch_bounds__(WG_THREADS, 2) cnn_wgrad_kernel(wgrad_args ar)
     }
 }
 
-// The gradient: the blocks' partial gradients of each layer added in block order.
-__global__ void cnn_grad_sum_kernel(wgrad_args ar, float *__restrict__ grads) {
+// The gradient: the blocks' partial gradients of each layer, added by 8 thread rows of 4 sums each
+// (one thread per weight waited 13 us for its chain of loads).
+constexpr int GS_ROWS = 8;
+__global__ void __launch_bounds__(32 * GS_ROWS)
+cnn_grad_sum_kernel(wgrad_args ar, float *__restrict__ grads) {
+    __shared__ float red[GS_ROWS][32];
     const wgrad_job jb = ar.job[blockIdx.y];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= jb.size) return;
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
     float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    int x = 0;
-    for (; x + 4 <= jb.blocks; x += 4)
+    if (i < jb.size) {
+        int x = row;
+        for (; x + 3 * GS_ROWS < jb.blocks; x += 4 * GS_ROWS)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] += jb.part[(int64_t)(x + k) * jb.size + i];
-    for (; x < jb.blocks; ++x) v[0] += jb.part[(int64_t)x * jb.size + i];
-    int64_t off = 0;
-    for (int l = 0; l < (int)blockIdx.y; ++l) off += ar.job[l].size;
-    grads[off + i] = (v[0] + v[1]) + (v[2] + v[3]);
+            for (int k = 0; k < 4; ++k) v[k] += jb.part[(int64_t)(x + k * GS_ROWS) * jb.size + i];
+        for (; x < jb.blocks; x += GS_ROWS) v[0] += jb.part[(int64_t)x * jb.size + i];
+    }
+    red[row][lane] = (v[0] + v[1]) + (v[2] + v[3]);
+    __syncthreads();
+    if (row == 0 && i < jb.size) {
+        float sum = red[0][lane];
+#pragma unroll
+        for (int r = 1; r < GS_ROWS; ++r) sum += red[r][lane];
+        int64_t off = 0;
+        for (int l = 0; l < (int)blockIdx.y; ++l) off += ar.job[l].size;
+        grads[off + i] = sum;
+    }
 }
 
 __global__ void cnn_round_kernel(const float *__restrict__ w, __nv_bfloat16 *__restrict__ wb,
@@ -1110,7 +1167,7 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
     n->d_m = reinterpret_cast<float *>(take(P * 4));
     n->d_v = reinterpret_cast<float *>(take(P * 4));
     n->d_wb = reinterpret_cast<__nv_bfloat16 *>(take(P * 2));
-    n->d_loss = reinterpret_cast<double *>(take(8));
+    n->d_loss = reinterpret_cast<double *>(take(8 + CNN_LAYERS * sizeof(int)));
     for (int l = 0; l < CNN_LAYERS; ++l) n->d_act[l] = reinterpret_cast<float *>(take(act * 4));
     n->d_act[CNN_LAYERS] = reinterpret_cast<float *>(take(logits * 4));
     for (float *&g : n->d_g) g = reinterpret_cast<float *>(take(act * 4));
@@ -1200,7 +1257,8 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
     if (!e) e = forward(ctx, n, d_features, B, nullptr);
-    if (!e) e = cudaMemsetAsync(n->d_loss, 0, sizeof(double), ctx->stream);
+    // the loss and the tile counters behind it
+    if (!e) e = cudaMemsetAsync(n->d_loss, 0, 8 + CNN_LAYERS * sizeof(int), ctx->stream);
     if (!e) {
         back_args ar{};
         ar.w1 = n->d_wb + n->w_off[1];
@@ -1233,6 +1291,7 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
         wgrad_args ar{};
         ar.logits = n->d_act[CNN_LAYERS];
         ar.labels = d_labels;
+        ar.next = reinterpret_cast<int *>(n->d_loss + 1);
         ar.wpos = pos_weight;
         ar.n = (int64_t)B * T;
         ar.B = B;
@@ -1266,8 +1325,8 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
             e = cudaGetLastError();
         }
         if (!e) {
-            dim3 grid((unsigned)((WG_PART + 127) / 128), CNN_LAYERS);
-            cnn_grad_sum_kernel<<<grid, 128, 0, ctx->stream>>>(ar, n->d_grads);
+            dim3 grid((unsigned)((WG_PART + 31) / 32), CNN_LAYERS);
+            cnn_grad_sum_kernel<<<grid, 32 * GS_ROWS, 0, ctx->stream>>>(ar, n->d_grads);
             ctx->launches++;
             e = cudaGetLastError();
         }
