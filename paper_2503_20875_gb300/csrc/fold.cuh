@@ -787,26 +787,38 @@ __device__ void build_pack_list(fold_smem &sm, int g0) {
     if (lane == 0) sm.pack_n = n;
 }
 
-// Run by the producer warp's first lane alone: per tile of H listed durations and per live
-// epoch, one strip of H segments (one bulk copy per row, one barrier arrival for all).
+// Run by the whole producer warp: per tile of H listed durations and per live epoch, one strip
+// of H segments, a bulk copy per row and one barrier arrival for all. Each lane issues its rows'
+// copies (one lane issuing up to 12 after one another, at about 50 clocks each, took longer than
+// the consumers' epoch).
 __device__ void produce_packed(fold_smem &sm, uint32_t ring0, const fold_table &tb, int Tp, int H,
                                int seg, ring &rg) {
+    const int lane = threadIdx.x & 31;
+    rg.par = __shfl_sync(0xFFFFFFFFu, rg.par, 0);  // (the other paths' copies are the first lane's)
     const int nJ = sm.pack_n;
     const int nE = live_epochs(tb, tb.Es, sm.it.I, 0);
     const uint32_t seg_bytes = (uint32_t)seg * (uint32_t)sizeof(float2);
     for (int t0 = 0; t0 < nJ; t0 += H) {
         const int nr = min(H, nJ - t0);
+        const float2 *row =
+            sm.it.ab + (int64_t)sm.pack_j[min(t0 + lane, nJ - 1)] * sm.it.ld;  // of lane h < 32
         for (int e = 0; e < nE; ++e) {
-            if (!producer_wait(sm, &sm.empty[rg.stage], rg.parity() ^ 1u)) return;
             const int a = tb.lo(e) & ~1;
             const uint32_t bytes = (uint32_t)(((tb.hi(e) + Tp - a) + 1) & ~1) * (uint32_t)sizeof(float2);
             const uint32_t dst = ring0 + rg.stage * rg.bytes;
-            fence_proxy_async();
-            mbar_expect_tx(&sm.full[rg.stage], bytes * (uint32_t)nr);
-            for (int h = 0; h < nr; ++h) {
-                const float2 *src = sm.it.ab + (int64_t)sm.pack_j[t0 + h] * sm.it.ld + a;
-                bulk_load_s(dst + (uint32_t)h * seg_bytes, src, bytes, &sm.full[rg.stage]);
+            bool ok = true;
+            if (lane == 0) {
+                ok = producer_wait(sm, &sm.empty[rg.stage], rg.parity() ^ 1u);
+                if (ok) mbar_expect_tx(&sm.full[rg.stage], bytes * (uint32_t)nr);
             }
+            if (!__shfl_sync(0xFFFFFFFFu, (int)ok, 0)) return;
+            fence_proxy_async();
+            if (lane < nr)
+                bulk_load_s(dst + (uint32_t)lane * seg_bytes, row + a, bytes, &sm.full[rg.stage]);
+            for (int h = lane + 32; h < nr; h += 32)
+                bulk_load_s(dst + (uint32_t)h * seg_bytes,
+                            sm.it.ab + (int64_t)sm.pack_j[t0 + h] * sm.it.ld + a, bytes,
+                            &sm.full[rg.stage]);
             rg.next();
         }
     }
@@ -1042,8 +1054,7 @@ __device__ void fold_subgroup(fold_smem &sm, uint32_t ring0, const fold_table &t
         // duration-packed (no block barrier, as the main path)
         if constexpr (GS >= 4) {
             if (producer) {
-                if ((threadIdx.x & 31) == 0) produce_packed(sm, ring0, tb, Tp, H, seg, rg);
-                __syncwarp();
+                produce_packed(sm, ring0, tb, Tp, H, seg, rg);
             } else {
                 consume_packed<GS, R, W, KAHAN>(sm, ring0, tb, g0, Tp, H, seg, rg);
             }
