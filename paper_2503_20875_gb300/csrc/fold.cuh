@@ -307,6 +307,10 @@ __device__ __forceinline__ void load_factors(const fold_smem &sm, int g0, float 
     }
 }
 
+__device__ __forceinline__ float load_factor(const fold_smem &sm, int g) {
+    return __int_as_float(*(const volatile int *)&sm.factor[g]);
+}
+
 // Offer slot g the best window of each lane of a warp (called by whole warps): 2 LR = lr2 at
 // flat index at; a lane without one passes lr2 < 0. The larger LR stays, on equal LR the smaller
 // flat index (make_key).
@@ -458,8 +462,7 @@ __device__ __forceinline__ bool consume_epochs(fold_smem &sm, const fold_table &
 template <int GS, int R, int W, bool KAHAN, bool SHORT>
 __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb, int g0, int j,
                                              int i0, int nE, unsigned use, bool all_used,
-                                             int nmin, uint32_t mine, ring &rg) {
-    constexpr int T = FT_THREADS * R;
+                                             uint32_t mine, ring &rg) {
     const int c = threadIdx.x;
     uint64_t acc[GS][R];
     uint64_t cmp[KAHAN ? GS : 1][KAHAN ? R : 1];  // minus the Kahan compensation
@@ -534,9 +537,12 @@ __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb
                      : consume_epochs<GS, R, W, KAHAN, false>(sm, tb, nE, use, mine, acc, cmp, rg);
         if (!ok) return false;
     }
-    // 2 LR = SA^2 / SB per (period, phase). Whole tiles (nmin: the phases every used period
-    // has) first run the candidate test over all their windows.
-    float m = i0 + T > nmin ? 1.0f : -1.0f;  // a ragged tile takes the exact comparisons
+    // 2 LR = SA^2 / SB per (period, phase): the candidate test over all the tile's windows
+    // (also those past a period's last phase, which the exact branch leaves out), then the exact
+    // values of the periods that have candidates. The exact branch takes a few thousand clocks: in
+    // every period's name, or for every tile that reaches past some period's last phase (the last
+    // one of each row), it was a tenth of the time of short work items.
+    float m = -1.0f;
     float h[GS];
     load_factors<GS>(sm, g0, h);
 #pragma unroll
@@ -556,6 +562,18 @@ __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb
 #pragma unroll
         for (int gg = 0; gg < GS; ++gg) {
             if (!((use >> gg) & 1u)) continue;
+            // the periods with a candidate only
+            const float hg = load_factor(sm, g0 + gg);
+            float mg = -1.0f;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                uint64_t v = acc[gg][r];
+                if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
+                float x, y;
+                split_pair(v, x, y);
+                mg = fmaxf(mg, fmaf(x, x, -(hg * y)));
+            }
+            if (!__any_sync(0xFFFFFFFFu, mg > 0.0f)) continue;
             const int nph = sm.nph[g0 + gg];
             float lr2 = -1.0f;
             uint32_t at = 0u;
@@ -579,17 +597,17 @@ __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb
 template <int GS, int R, int W, bool KAHAN, int RL>
 __device__ __forceinline__ bool consume_tile_rows(int rows, fold_smem &sm, const fold_table &tb,
                                                   int g0, int j, int i0, int nE, unsigned use,
-                                                  bool all_used, int nmin, uint32_t mine,
+                                                  bool all_used, uint32_t mine,
                                                   ring &rg) {
     if constexpr (RL > 1 && GS >= 4) {
         if (rows < RL)
             return consume_tile_rows<GS, R, W, KAHAN, RL - 1>(rows, sm, tb, g0, j, i0, nE, use,
-                                                              all_used, nmin, mine, rg);
+                                                              all_used, mine, rg);
     }
     return nE <= 3 ? consume_tile<GS, RL, W, KAHAN, true>(sm, tb, g0, j, i0, nE, use, all_used,
-                                                          nmin, mine, rg)
+                                                          mine, rg)
                    : consume_tile<GS, RL, W, KAHAN, false>(sm, tb, g0, j, i0, nE, use, all_used,
-                                                           nmin, mine, rg);
+                                                           mine, rg);
 }
 
 template <int GS, int R, int W, bool KAHAN>
@@ -602,17 +620,13 @@ __device__ void consume_main(fold_smem &sm, uint32_t ring0, const fold_table &tb
         const unsigned use = period_use<GS>(sm, g0, j);
         if (!use) continue;
         const bool all_used = use == (1u << GS) - 1u;
-        int nmin = nph_sub;  // phases every used period has
-#pragma unroll
-        for (int gg = 0; gg < GS; ++gg)
-            if ((use >> gg) & 1u) nmin = min(nmin, sm.nph[g0 + gg]);
         int nE = tb.Es;
         for (int i0 = 0; i0 < nph_sub; i0 += T) {
             nE = live_epochs(tb, nE, sm.it.I, i0);
             // (a wait that gave up ends the path at once: the main path has no block barrier,
             // so every thread still meets the caller's next one)
             const bool ok = consume_tile_rows<GS, R, W, KAHAN, R>(
-                tile_rows<GS, R>(nph_sub - i0), sm, tb, g0, j, i0, nE, use, all_used, nmin, mine,
+                tile_rows<GS, R>(nph_sub - i0), sm, tb, g0, j, i0, nE, use, all_used, mine,
                 rg);
             if (!ok) return;
         }
@@ -639,18 +653,20 @@ __device__ void produce_sliced(fold_smem &sm, uint32_t ring0, const fold_table &
     constexpr int T = FT_THREADS * R;
     const int H = T / Tp;
     const int I = sm.it.I;
-    const bool leader = (threadIdx.x & 31) == 0;
+    const int lane = threadIdx.x & 31;
     for (int j = sm.it.jlo; j < sm.it.jhi; ++j) {
         const unsigned use = period_use<GS>(sm, g0, j);
         if (!use) continue;
         for (int s = 0; live_epoch(tb, s * H, I); ++s) {
+            // the strip's end, a slice's epoch per lane
+            const int e0 = s * H;
+            int end = 0;
+            for (int h = lane; h < H; h += 32)
+                if (live_epoch(tb, e0 + h, I)) end = max(end, tb.hi(e0 + h) + Tp);
+            end = __reduce_max_sync(0xFFFFFFFFu, end);
             // (after an abort this only keeps the loop, and the barriers below, in step)
-            if (leader && producer_wait(sm, &sm.empty[rg.stage], rg.parity() ^ 1u)) {
-                const int e0 = s * H;
+            if (lane == 0 && producer_wait(sm, &sm.empty[rg.stage], rg.parity() ^ 1u)) {
                 const int a = tb.lo(e0) & ~1;
-                int end = 0;
-                for (int h = 0; h < H; ++h)
-                    if (live_epoch(tb, e0 + h, I)) end = max(end, tb.hi(e0 + h) + Tp);
                 issue_copy(sm, ring0, rg, j, a, ((end - a) + 1) & ~1);
             }
             __syncwarp();
@@ -746,7 +762,7 @@ __device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part,
                 split_pair(v, x, y);
                 take_max(x, y, (uint32_t)j * (uint32_t)I + (uint32_t)phi, lr2, at);
             }
-            if (__any_sync(0xFFFFFFFFu, lr2 > __int_as_float(*(volatile int *)&sm.factor[g0 + gg])))
+            if (__any_sync(0xFFFFFFFFu, lr2 > load_factor(sm, g0 + gg)))
                 offer_best(sm, g0 + gg, lr2, at);
             block_sync();
         }
@@ -824,104 +840,140 @@ __device__ void produce_packed(fold_smem &sm, uint32_t ring0, const fold_table &
     }
 }
 
+// One tile of listed durations t0 .. t0 + nr - 1, whose nr Tp lanes with work are within the
+// first R rows of FT_THREADS lanes.
 template <int GS, int R, int W, bool KAHAN>
-__device__ void consume_packed(fold_smem &sm, uint32_t ring0, const fold_table &tb,
-                               int g0, int Tp, int H, int seg, ring &rg) {
-    const int c = threadIdx.x;
-    const int nJ = sm.pack_n;
+__device__ __forceinline__ bool packed_tile(fold_smem &sm, uint32_t ring0, const fold_table &tb,
+                                            int g0, int Tp, int H, int seg, int t0, int nr, int nE,
+                                            ring &rg) {
     const uint32_t I = (uint32_t)sm.it.I;
-    const int nE = live_epochs(tb, tb.Es, sm.it.I, 0);
-    int row[R], ph[R];
     uint32_t base[R];  // the lane's cell in its row's segment (bytes from the strip's start)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int L = c + r * FT_THREADS;
-        row[r] = L / Tp;
-        ph[r] = L - row[r] * Tp;
-        base[r] = row[r] < H ? ((uint32_t)row[r] * (uint32_t)seg + (uint32_t)ph[r]) *
-                                   (uint32_t)sizeof(float2)
-                             : 0u;  // idle lane: reads row 0, never used
+        const int L = threadIdx.x + r * FT_THREADS, row = L / Tp;
+        base[r] = row < H ? (uint32_t)(row * seg + L - row * Tp) * (uint32_t)sizeof(float2)
+                          : 0u;  // idle lane: reads row 0, never used
     }
+    uint64_t acc[GS][R];
+    uint64_t cmp[KAHAN ? GS : 1][KAHAN ? R : 1];
+    // epoch 0: every period's cell is its phase cell (o_0 = 0), one load for all
+    if (!fold_wait(sm, &sm.full[rg.stage], rg.parity())) return false;
+    {
+        const uint32_t a = ring0 + rg.stage * rg.bytes;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const uint64_t v = lds_pair(a + base[r]);
+#pragma unroll
+            for (int gg = 0; gg < GS; ++gg) acc[gg][r] = v;
+        }
+        mbar_arrive(&sm.empty[rg.stage]);
+    }
+    rg.next();
+    if constexpr (KAHAN) {
+#pragma unroll
+        for (int gg = 0; gg < GS; ++gg)
+#pragma unroll
+            for (int r = 0; r < R; ++r) cmp[gg][r] = 0ull;
+    }
+    for (int e = 1; e < nE; ++e) {
+        if (!fold_wait(sm, &sm.full[rg.stage], rg.parity())) return false;
+        const uint32_t a = ring0 + rg.stage * rg.bytes;
+        epoch_offsets<GS, W> off;
+        off.load(tb.off + (uint32_t)(e * GS * W));
+        uint32_t ar[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) ar[r] = a + base[r];
+#pragma unroll
+        for (int gg = 0; gg < GS; ++gg) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const uint64_t v = lds_pair(ar[r] + off[gg]);
+                if constexpr (KAHAN)
+                    kahan_add_pair(acc[gg][r], cmp[gg][r], v);
+                else
+                    add_pair(acc[gg][r], v);
+            }
+        }
+        mbar_arrive(&sm.empty[rg.stage]);
+        rg.next();
+    }
+    // maxima, the lane's windows in (duration, phase) order
+    unsigned use[R];
+    float m = -1.0f;
+    float h[GS];
+    load_factors<GS>(sm, g0, h);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int row = (int)(threadIdx.x + r * FT_THREADS) / Tp;
+        use[r] = row < nr ? sm.pack_use[t0 + row] : 0u;
+    }
+#pragma unroll
+    for (int gg = 0; gg < GS; ++gg) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            uint64_t v = acc[gg][r];
+            if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
+            float x, y;
+            split_pair(v, x, y);
+            if ((use[r] >> gg) & 1u) m = fmaxf(m, fmaf(x, x, -(h[gg] * y)));
+        }
+    }
+    if (!__any_sync(0xFFFFFFFFu, m > 0.0f)) return true;
+#pragma unroll
+    for (int gg = 0; gg < GS; ++gg) {
+        const float hg = load_factor(sm, g0 + gg);
+        float mg = -1.0f;  // the periods with a candidate only
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            uint64_t v = acc[gg][r];
+            if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
+            float x, y;
+            split_pair(v, x, y);
+            if ((use[r] >> gg) & 1u) mg = fmaxf(mg, fmaf(x, x, -(hg * y)));
+        }
+        if (!__any_sync(0xFFFFFFFFu, mg > 0.0f)) continue;
+        float lr2 = -1.0f;
+        uint32_t at = 0u;
+        const int nph = sm.nph[g0 + gg];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int L = threadIdx.x + r * FT_THREADS, row = L / Tp, ph = L - row * Tp;
+            if (!((use[r] >> gg) & 1u) || ph >= nph) continue;
+            uint64_t v = acc[gg][r];
+            if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
+            float x, y;
+            split_pair(v, x, y);
+            take_max(x, y, (uint32_t)sm.pack_j[t0 + row] * I + (uint32_t)ph, lr2, at);
+        }
+        offer_best(sm, g0 + gg, lr2, at);
+    }
+    return true;
+}
+
+// The variant with as many rows of lanes as the tile has work for (rows <= R): lanes past the
+// last row load nothing.
+template <int GS, int R, int W, bool KAHAN>
+__device__ __forceinline__ bool packed_tile_rows(int rows, fold_smem &sm, uint32_t ring0,
+                                                 const fold_table &tb, int g0, int Tp, int H,
+                                                 int seg, int t0, int nr, int nE, ring &rg) {
+    if constexpr (R > 1 && !KAHAN) {  // (the compensated form's tiles are half as wide)
+        if (rows < R)
+            return packed_tile_rows<GS, R - 1, W, KAHAN>(rows, sm, ring0, tb, g0, Tp, H, seg, t0,
+                                                         nr, nE, rg);
+    }
+    return packed_tile<GS, R, W, KAHAN>(sm, ring0, tb, g0, Tp, H, seg, t0, nr, nE, rg);
+}
+
+template <int GS, int R, int W, bool KAHAN>
+__device__ void consume_packed(fold_smem &sm, uint32_t ring0, const fold_table &tb, int g0, int Tp,
+                               int H, int seg, ring &rg) {
+    const int nJ = sm.pack_n;
+    const int nE = live_epochs(tb, tb.Es, sm.it.I, 0);
     for (int t0 = 0; t0 < nJ; t0 += H) {
         const int nr = min(H, nJ - t0);
-        uint64_t acc[GS][R];
-        uint64_t cmp[KAHAN ? GS : 1][KAHAN ? R : 1];
-        // epoch 0: every period's cell is its phase cell (o_0 = 0), one load for all
-        if (!fold_wait(sm, &sm.full[rg.stage], rg.parity())) return;
-        {
-            const uint32_t a = ring0 + rg.stage * rg.bytes;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const uint64_t v = lds_pair(a + base[r]);
-#pragma unroll
-                for (int gg = 0; gg < GS; ++gg) acc[gg][r] = v;
-            }
-            mbar_arrive(&sm.empty[rg.stage]);
-        }
-        rg.next();
-        if constexpr (KAHAN) {
-#pragma unroll
-            for (int gg = 0; gg < GS; ++gg)
-#pragma unroll
-                for (int r = 0; r < R; ++r) cmp[gg][r] = 0ull;
-        }
-        for (int e = 1; e < nE; ++e) {
-            if (!fold_wait(sm, &sm.full[rg.stage], rg.parity())) return;
-            const uint32_t a = ring0 + rg.stage * rg.bytes;
-            epoch_offsets<GS, W> off;
-            off.load(tb.off + (uint32_t)(e * GS * W));
-            uint32_t ar[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) ar[r] = a + base[r];
-#pragma unroll
-            for (int gg = 0; gg < GS; ++gg) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const uint64_t v = lds_pair(ar[r] + off[gg]);
-                    if constexpr (KAHAN)
-                        kahan_add_pair(acc[gg][r], cmp[gg][r], v);
-                    else
-                        add_pair(acc[gg][r], v);
-                }
-            }
-            mbar_arrive(&sm.empty[rg.stage]);
-            rg.next();
-        }
-        // maxima, the lane's windows in (duration, phase) order
-        unsigned use[R];
-        float m = -1.0f;
-#pragma unroll
-        for (int r = 0; r < R; ++r) use[r] = row[r] < nr ? sm.pack_use[t0 + row[r]] : 0u;
-        float h[GS];
-        load_factors<GS>(sm, g0, h);
-#pragma unroll
-        for (int gg = 0; gg < GS; ++gg) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                uint64_t v = acc[gg][r];
-                if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
-                float x, y;
-                split_pair(v, x, y);
-                if ((use[r] >> gg) & 1u) m = fmaxf(m, fmaf(x, x, -(h[gg] * y)));
-            }
-        }
-        if (!__any_sync(0xFFFFFFFFu, m > 0.0f)) continue;
-#pragma unroll
-        for (int gg = 0; gg < GS; ++gg) {
-            float lr2 = -1.0f;
-            uint32_t at = 0u;
-            const int nph = sm.nph[g0 + gg];
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (!((use[r] >> gg) & 1u) || ph[r] >= nph) continue;
-                uint64_t v = acc[gg][r];
-                if constexpr (KAHAN) add_pair(v, cmp[gg][r]);
-                float x, y;
-                split_pair(v, x, y);
-                take_max(x, y, (uint32_t)sm.pack_j[t0 + row[r]] * I + (uint32_t)ph[r], lr2, at);
-            }
-            offer_best(sm, g0 + gg, lr2, at);
-        }
+        const int rows = (nr * Tp + FT_THREADS - 1) / FT_THREADS;
+        if (!packed_tile_rows<GS, R, W, KAHAN>(rows, sm, ring0, tb, g0, Tp, H, seg, t0, nr, nE, rg))
+            return;
     }
 }
 
