@@ -40,10 +40,14 @@ __device__ __forceinline__ void add2(float2 &acc, float2 v) {
 #endif
 }
 
-// d = a - b elementwise with one packed FP32x2 subtract.
+// (-1, -1) as a packed FP32 pair.
+constexpr unsigned long long MINUS_ONES = 0xBF800000BF800000ull;
+constexpr unsigned long long ONES = 0x3F8000003F800000ull;
+
+// d = a - b elementwise: one packed multiply-add by -1 (the same rounding as a subtraction).
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
     unsigned long long d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack2(b)), "l"(MINUS_ONES), "l"(pack2(a)));
     return unpack2(d);
 }
 

@@ -93,14 +93,16 @@ __device__ __forceinline__ uint64_t sum_pair(uint64_t a, uint64_t b) {
 }
 
 // Kahan-compensated s += v on packed pairs; nc holds minus the running compensation:
-// y = v + nc, t = s + y, nc = y - (t - s), s = t.
+// y = v + nc, t = s + y, nc = y - (t - s), s = t. The differences are multiply-adds by -1 (the
+// same single rounding of the exact difference). t is worked out again into s's registers: s and
+// t live at the same time, so that a loop over s = t moved two registers per step.
 __device__ __forceinline__ void kahan_add_pair(uint64_t &s, uint64_t &nc, uint64_t v) {
     uint64_t y, t, d;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(v), "l"(nc));
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(s), "l"(y));
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(t), "l"(s));
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(nc) : "l"(y), "l"(d));
-    s = t;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(s), "l"(MINUS_ONES), "l"(t));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(nc) : "l"(d), "l"(MINUS_ONES), "l"(y));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s) : "l"(y), "l"(ONES));  // t, in place
 }
 
 __device__ __forceinline__ void split_pair(uint64_t v, float &x, float &y) {
