@@ -57,6 +57,7 @@ constexpr int NET_XROWS = NET_ROWS + 8;    // rows held: 8 more for the last tap
 constexpr int NET_OUT = NET_ROWS - 24;     // logits per tile
 constexpr int NET_THREADS = 256;
 constexpr int NET_GRP = 4;                 // accumulators of a sum
+constexpr int NET_AHEAD = 2;               // input items a thread reads ahead (any tile has as many)
 constexpr int NET_UNIT = NET_XROWS * 16;   // bytes of one 8-channel unit of all rows
 constexpr int NET_PART = 4 * NET_UNIT;     // bytes of one BF16 part (32 channels)
 constexpr int NET_ACT3_LD = 260;           // floats per channel row of the last activation
@@ -148,6 +149,23 @@ __device__ __forceinline__ void net_tmem_wait(float (&v)[16]) {
                  : "memory");
 }
 
+// Sixteen channels of a row: the sums of the NET_GRP accumulators, in pairs.
+__device__ __forceinline__ void net_sums(float (&v)[16], uint32_t taddr) {
+    float o[16], w[16];
+    net_tmem_load(v, taddr);
+    net_tmem_load(o, taddr + CNN_C);
+    net_tmem_wait(v);
+    net_tmem_wait(o);
+    net_tmem_load(w, taddr + 2 * CNN_C);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] += o[c];
+    net_tmem_load(o, taddr + 3 * CNN_C);
+    net_tmem_wait(w);
+    net_tmem_wait(o);
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] += w[c] + o[c];
+}
+
 // Eight channels of one row as three BF16 parts (the leading, middle and last 8 bits of each
 // value: exact) into the 16-byte slot at `at` of every part.
 __device__ __forceinline__ void net_store_row(uint32_t at, const float *v) {
@@ -226,22 +244,32 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tm = s_tmem;
 
+    // item `it` of a tile's input: row it % NET_XROWS (bin t0 - 16 + row), channels 8 u .. 8 u + 7,
+    // u = it / NET_XROWS
+    auto read_item = [&](int tile, int it, float (&v)[8]) {
+        const int b = tile / tiles_per_curve, u = it / NET_XROWS;
+        const int t = (tile - b * tiles_per_curve) * NET_OUT - 16 + it - u * NET_XROWS;
+        const float *fb = features + (int64_t)b * cin * T + t;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int ci = u * 8 + e;
+            v[e] = t >= 0 && t < T && ci < cin ? fb[(int64_t)ci * T] : 0.0f;
+        }
+    };
+    const int items = NET_XROWS * units1;
+    float ahead[NET_AHEAD][8];  // the first items of the next tile, read under the last layer
+    if (blockIdx.x < n_tiles)
+#pragma unroll
+        for (int x = 0; x < NET_AHEAD; ++x) read_item(blockIdx.x, tid + x * NET_THREADS, ahead[x]);
     uint32_t phase = 0;
     bool failed = false;
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int b = tile / tiles_per_curve;
         const int t0 = (tile - b * tiles_per_curve) * NET_OUT;
-        // layer 0: log1p of the features, rows t0 - 16 + i
-        const float *fb = features + (int64_t)b * cin * T;
-        for (int it = tid; it < NET_XROWS * units1; it += NET_THREADS) {
+        // layer 0: log1p of the features
+        auto put_item = [&](int it, float (&v)[8]) {
             const int u = it / NET_XROWS, i = it - u * NET_XROWS;
             const int t = t0 - 16 + i;
-            float v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int ci = u * 8 + e;
-                v[e] = t >= 0 && t < T && ci < cin ? fb[(int64_t)ci * T + t] : 0.0f;
-            }
 #pragma unroll
             for (int e = 0; e < 8; ++e) v[e] = log1pf(fmaxf(v[e], 0.0f));
             if (STORE && t >= t0 && t < T && t < t0 + NET_OUT)
@@ -250,6 +278,13 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
                     if (u * 8 + e < cin)
                         net.act[0][((int64_t)b * cin + u * 8 + e) * T + t] = v[e];
             net_store_row(x0 + (uint32_t)(u * NET_UNIT + i * 16), v);
+        };
+#pragma unroll
+        for (int x = 0; x < NET_AHEAD; ++x) put_item(tid + x * NET_THREADS, ahead[x]);
+        for (int it = tid + NET_AHEAD * NET_THREADS; it < items; it += NET_THREADS) {
+            float v[8];
+            read_item(tile, it, v);
+            put_item(it, v);
         }
         fence_proxy_async();
         __syncthreads();
@@ -270,6 +305,10 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
                 }
             }
             __syncwarp();
+            if (l == 2 && tile + (int)gridDim.x < n_tiles)
+#pragma unroll
+                for (int x = 0; x < NET_AHEAD; ++x)
+                    read_item(tile + gridDim.x, tid + x * NET_THREADS, ahead[x]);
             // epilogue: warps 0-3 the rows of block 0, warps 4-7 of block 1 (in place: the other
             // block's instructions read no row of this one). The last layer's FP32 activations
             // overlay the parts, so it waits for both blocks.
@@ -286,16 +325,8 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
             const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                float v[16], o[16];
-                net_tmem_load(v, src + h * 16);
-                net_tmem_wait(v);
-#pragma unroll
-                for (int g = 1; g < NET_GRP; ++g) {
-                    net_tmem_load(o, src + g * CNN_C + h * 16);
-                    net_tmem_wait(o);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] += o[c];
-                }
+                float v[16];
+                net_sums(v, src + h * 16);
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     const float a = fmaxf(v[c] + bias[l * CNN_C + h * 16 + c], 0.0f);
@@ -520,16 +551,8 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
             const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                float v[16], o[16];
-                net_tmem_load(v, src + h * 16);
-                net_tmem_wait(v);
-#pragma unroll
-                for (int g = 1; g < NET_GRP; ++g) {
-                    net_tmem_load(o, src + g * CNN_C + h * 16);
-                    net_tmem_wait(o);
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] += o[c];
-                }
+                float v[16];
+                net_sums(v, src + h * 16);
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     v[c] = (mask >> (h * 16 + c)) & 1u ? v[c] : 0.0f;

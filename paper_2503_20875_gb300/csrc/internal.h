@@ -70,7 +70,8 @@ struct cetra_plan {
     // linear kernel launch shape, chosen from p and the table lengths
     int lin_threads = 128, lin_kc = 0;
     size_t lin_smem = 0;
-    // device copies (owned)
+    // device copies (one owned allocation)
+    void *d_mem = nullptr;
     double *d_durations = nullptr;
     int32_t *d_win_a = nullptr, *d_win_len = nullptr, *d_win_padlen = nullptr;
     // linear-stage rows (duration, phase class) by decreasing window length: the kernel takes

@@ -208,52 +208,53 @@ int plan_build(cetra_ctx *ctx, const cetra_params *params, const double *time, c
     return CETRA_OK;
 }
 
-namespace {
-template <typename T>
-int upload(cetra_ctx *ctx, T **dst, const T *src, size_t n) {
-    *dst = nullptr;
-    if (n == 0) return CETRA_OK;
-    cudaError_t e = cudaMalloc((void **)dst, n * sizeof(T));
-    if (e != cudaSuccess) {
-        *dst = nullptr;
-        return set_error(ctx, CETRA_ENOMEM, std::string("plan upload: ") + cudaGetErrorString(e));
-    }
-    e = cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return set_error(ctx, CETRA_ECUDA, cudaGetErrorString(e));
-    return CETRA_OK;
-}
-}  // namespace
-
+// The plan's device tables, one allocation and one copy (seven of each took longer than a small
+// curve's search).
 int plan_upload(cetra_ctx *ctx, cetra_plan *plan) {
-    int rc;
-    if ((rc = upload(ctx, &plan->d_durations, plan->durations.data(), plan->durations.size())))
-        return rc;
-    if ((rc = upload(ctx, &plan->d_win_a, plan->win_a.data(), plan->win_a.size()))) return rc;
-    if ((rc = upload(ctx, &plan->d_win_len, plan->win_len.data(), plan->win_len.size()))) return rc;
-    if ((rc = upload(ctx, &plan->d_win_padlen, plan->win_padlen.data(), plan->win_padlen.size())))
-        return rc;
-    if ((rc = upload(ctx, &plan->d_win_off, plan->win_off.data(), plan->win_off.size()))) return rc;
     plan->lin_order.resize(plan->win_padlen.size());
     for (size_t x = 0; x < plan->lin_order.size(); ++x) plan->lin_order[x] = (int32_t)x;
     std::stable_sort(plan->lin_order.begin(), plan->lin_order.end(), [&](int32_t a, int32_t b) {
         return plan->win_padlen[(size_t)a] > plan->win_padlen[(size_t)b];
     });
-    if ((rc = upload(ctx, &plan->d_lin_order, plan->lin_order.data(), plan->lin_order.size())))
-        return rc;
-    if ((rc = upload(ctx, &plan->d_tables, plan->tables.data(), plan->tables.size()))) return rc;
-    cudaError_t e = linear_configure(plan, ctx);
+    std::vector<unsigned char> host;
+    auto add = [&](const void *src, size_t bytes) {
+        const size_t at = host.size();
+        const unsigned char *b = static_cast<const unsigned char *>(src);
+        host.insert(host.end(), b, b + bytes);
+        host.resize((host.size() + 255) & ~(size_t)255);
+        return at;
+    };
+    auto bytes = [](const auto &v) { return v.size() * sizeof(v[0]); };
+    const size_t o_tab = add(plan->tables.data(), bytes(plan->tables));
+    const size_t o_dur = add(plan->durations.data(), bytes(plan->durations));
+    const size_t o_off = add(plan->win_off.data(), bytes(plan->win_off));
+    const size_t o_a = add(plan->win_a.data(), bytes(plan->win_a));
+    const size_t o_len = add(plan->win_len.data(), bytes(plan->win_len));
+    const size_t o_pad = add(plan->win_padlen.data(), bytes(plan->win_padlen));
+    const size_t o_ord = add(plan->lin_order.data(), bytes(plan->lin_order));
+    cudaError_t e = cudaMalloc(&plan->d_mem, host.size());
+    if (e != cudaSuccess) {
+        plan->d_mem = nullptr;
+        return set_error(ctx, CETRA_ENOMEM, std::string("plan upload: ") + cudaGetErrorString(e));
+    }
+    e = cudaMemcpy(plan->d_mem, host.data(), host.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return set_error(ctx, CETRA_ECUDA, cudaGetErrorString(e));
+    char *base = static_cast<char *>(plan->d_mem);
+    plan->d_tables = reinterpret_cast<float2 *>(base + o_tab);
+    plan->d_durations = reinterpret_cast<double *>(base + o_dur);
+    plan->d_win_off = reinterpret_cast<int64_t *>(base + o_off);
+    plan->d_win_a = reinterpret_cast<int32_t *>(base + o_a);
+    plan->d_win_len = reinterpret_cast<int32_t *>(base + o_len);
+    plan->d_win_padlen = reinterpret_cast<int32_t *>(base + o_pad);
+    plan->d_lin_order = reinterpret_cast<int32_t *>(base + o_ord);
+    e = linear_configure(plan, ctx);
     if (e != cudaSuccess) return set_error(ctx, CETRA_ECUDA, cudaGetErrorString(e));
     return CETRA_OK;
 }
 
 void plan_free_device(cetra_plan *plan) {
-    cudaFree(plan->d_durations);
-    cudaFree(plan->d_win_a);
-    cudaFree(plan->d_win_len);
-    cudaFree(plan->d_win_padlen);
-    cudaFree(plan->d_win_off);
-    cudaFree(plan->d_lin_order);
-    cudaFree(plan->d_tables);
+    cudaFree(plan->d_mem);
+    plan->d_mem = nullptr;
     plan->d_durations = nullptr;
     plan->d_win_a = plan->d_win_len = plan->d_win_padlen = nullptr;
     plan->d_win_off = nullptr;
