@@ -23,7 +23,6 @@
 namespace {
 
 constexpr int CNN_K = 9;           // kernel width
-constexpr int CNN_HALF = CNN_K / 2;
 constexpr int CNN_C = 32;          // hidden channels
 constexpr int CNN_LAYERS = 4;
 constexpr size_t kCombSmemMax = 98 * 1024;  // maps up to 24,576 bins (+ 512 cells) are staged
@@ -42,18 +41,19 @@ constexpr size_t kCombSmemMax = 98 * 1024;  // maps up to 24,576 bins (+ 512 cel
 // Precision: the weights are BF16 values; an FP32 activation is the exact sum of three BF16
 // parts (its leading 8, middle 8 and last 8 bits), so three products with the same weight give
 // the FP32 product exactly. The tensor core's accumulator truncates, so a sum is kept in NET_GRP
-// accumulators (taps 0-1, 2-3, 4-5, 6-8; each takes its last and middle parts first), which are
-// added in FP32. Measured error of the probabilities against 64 bits: see cnn_forward.
+// accumulators (taps 0 and 2, 1 and 3, 4, 6 and 8, 5 and 7; each takes its last and middle parts
+// first), which are added in FP32. Measured error of the probabilities against 64 bits: see cnn_forward.
 //
-// Halo: layer l's row r is bin t0 - 16 + 4 l + r. A tile computes NET_ROWS = 256 rows of the
-// first three layers in place (rows past the last valid one are never used): 256, 248, 240
-// valid rows, then NET_OUT = 232 logits. Rows outside [0, T) are zero (zero padding).
+// Halo: layer l's row r is bin t0 - 16 + 4 l + r. A tile computes NET_ROWS = 254 rows of the
+// first three layers in place (rows past the last valid one are never used): 254, 246, 238
+// valid rows, then NET_OUT = 230 logits. Rows outside [0, T) are zero (zero padding).
 //
-// Bound: the shared-memory reads of the activation operand (4 KB, 32 clocks per instruction,
-// against 16 of arithmetic): 270 instructions per tile at 16 durations. Two blocks per SM, so
-// that one's epilogue runs under the other's matrix instructions.
-constexpr int NET_ROWS = 256;              // rows computed per layer (two M = 128 blocks)
-constexpr int NET_XROWS = NET_ROWS + 8;    // rows held: 8 more for the last tap
+// Bound: reading the activation operand from shared memory (4 KB per instruction): 150
+// instructions per tile at 16 durations. Two blocks per SM, so that one's epilogue runs under the
+// other's matrix instructions.
+constexpr int NET_BLOCK = 127;             // rows a block of 128 completes (see net_layer_mma)
+constexpr int NET_ROWS = 2 * NET_BLOCK;    // rows computed per layer
+constexpr int NET_XROWS = 264;             // rows held: 8 more for the last tap, whole groups of 8
 constexpr int NET_OUT = NET_ROWS - 24;     // logits per tile
 constexpr int NET_THREADS = 256;
 constexpr int NET_GRP = 4;                 // accumulators of a sum
@@ -62,14 +62,22 @@ constexpr int NET_UNIT = NET_XROWS * 16;   // bytes of one 8-channel unit of all
 constexpr int NET_PART = 4 * NET_UNIT;     // bytes of one BF16 part (32 channels)
 constexpr int NET_ACT3_LD = 260;           // floats per channel row of the last activation
 constexpr int NET_TMEM_COLS = 2 * NET_GRP * CNN_C;  // 256
-static_assert(3 * NET_PART >= CNN_C * NET_ACT3_LD * 4 + 4 * NET_ROWS * 4, "activation reuse");
+constexpr int NET_PLD = 256;               // partial logits per channel group
+static_assert(3 * NET_PART >= CNN_C * NET_ACT3_LD * 4 + 4 * NET_PLD * 4, "activation reuse");
 
 __host__ __device__ constexpr int net_units(int cin) { return (cin + 15) / 16 * 2; }
-// bytes of the BF16 weights of a layer with `units` input units: [tap][unit][co][8 ci]
+// bytes of the BF16 weights of a layer with `units` input units: taps 0-7 in pairs
+// [pair][unit][tap of the pair][co][8 ci], then tap 8 [unit][co][8 ci]
 __host__ __device__ constexpr int net_wbytes(int units) { return CNN_K * units * CNN_C * 16; }
 inline size_t net_smem(int cin) {
     return (size_t)3 * NET_PART + net_wbytes(net_units(cin)) + 2 * net_wbytes(4) +
            (CNN_C * CNN_K + 4 * CNN_C) * sizeof(float);
+}
+
+// Place of weight (tap k, unit u, co, element e) in them.
+__device__ __forceinline__ int net_wplace(int units, int k, int u, int co, int e) {
+    return k < 8 ? (((k >> 1) * units + u) * 64 + (k & 1) * CNN_C + co) * 8 + e
+                 : (4 * units * 64 + u * CNN_C + co) * 8 + e;
 }
 
 struct net_layers {
@@ -85,25 +93,35 @@ __device__ __forceinline__ uint32_t net_desc_lo(uint32_t addr, uint32_t unit_byt
     return ((addr >> 4) & 0x3FFFu) | ((unit_bytes >> 4) << 16);
 }
 
-// kind::f16: FP32 accumulator, BF16 operands, both K-major, M = 128, N = 32.
-constexpr uint32_t NET_IDESC =
-    (1u << 4) | (1u << 7) | (1u << 10) | ((CNN_C / 8) << 17) | ((128 / 16) << 24);
+// kind::f16: FP32 accumulator, BF16 operands, both K-major, M = 128, N = 32 or 64.
+__host__ __device__ constexpr uint32_t net_idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n / 8) << 17) | ((128u / 16) << 24);
+}
 
-__device__ __forceinline__ void net_mma(uint32_t d, uint64_t a, uint64_t b, bool add) {
+__device__ __forceinline__ void net_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+                                        bool add) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(NET_IDESC), "r"((uint32_t)add)
+        "l"(a), "l"(b), "r"(idesc), "r"((uint32_t)add)
         : "memory");
 }
-// The matrix instructions of one layer for one block of 128 rows (one thread): a_lo, b_lo are
-// the low words of the operands' descriptors at tap 0, unit 0, part 0. Consecutive instructions
-// go to different accumulators, and every offset is a constant of the unrolled code: with one
-// accumulator after the other and offsets worked out in the loop the instructions were issued
-// three times further apart (256 curves x 16 durations: 510 us against 297).
+// The matrix instructions of one layer for one block of 128 rows (one thread): a_lo, w are the
+// low word of the activations' descriptor at tap 0, unit 0, part 0, and the weights' address.
+//
+// Reading the activations is the bound, so an instruction takes two taps: N = 64 are the 32
+// output channels of taps 2 p and 2 p + 1, both on the rows of tap 2 p, and the second tap's sums
+// belong one row further down: out[r] = E0[r] + E1[r + 1] (net_sums). A block of 128 rows
+// therefore completes 127. One tap per instruction: 291 us for 256 curves x 16 durations.
+// Accumulators: E0 and E1 of pairs 0-1 and of pairs 2-4 (columns 0, 32, 64, 96), four partial
+// sums of every output. Consecutive instructions go to different ones, and every offset is a
+// constant of the unrolled code (worked out in a loop, one accumulator after the other, the
+// instructions were three times further apart).
 template <int UNITS>
-__device__ __forceinline__ void net_layer_mma(uint32_t d, uint32_t a_lo, uint32_t b_lo) {
+__device__ __forceinline__ void net_layer_mma(uint32_t d, uint32_t a_lo, uint32_t w) {
     constexpr uint32_t hi = (128u >> 4) | (1u << 14);
+    const uint32_t b64 = net_desc_lo(w, 64 * 16);
+    const uint32_t b32 = net_desc_lo(w + 4 * UNITS * 64 * 16, CNN_C * 16);
 #pragma unroll
     for (int q = 2; q >= 0; --q)
 #pragma unroll
@@ -111,14 +129,20 @@ __device__ __forceinline__ void net_layer_mma(uint32_t d, uint32_t a_lo, uint32_
 #pragma unroll
             for (int u = 0; u < UNITS; u += 2)
 #pragma unroll
-                for (int g = 0; g < NET_GRP; ++g) {
-                    const int k = 2 * g + j;
-                    if (j == 2 && g < NET_GRP - 1) continue;  // the last group has three taps
-                    const uint64_t a =
-                        ((uint64_t)hi << 32) | (a_lo + (q * NET_PART + u * NET_UNIT + k * 16) / 16);
-                    const uint64_t b =
-                        ((uint64_t)hi << 32) | (b_lo + (k * UNITS + u) * CNN_C * 16 / 16);
-                    net_mma(d + g * CNN_C, a, b, q < 2 || j > 0 || u > 0);
+                for (int g = 0; g < 2; ++g) {
+                    if (g == 0 && j == 2) continue;  // pairs 0, 1 and 2, 3, 4 (tap 8 alone)
+                    const int pair = g == 0 ? j : 2 + j;
+                    const uint64_t a = ((uint64_t)hi << 32) |
+                                       (a_lo + (q * NET_PART + u * NET_UNIT + 2 * pair * 16) / 16);
+                    const bool add = q < 2 || j > 0 || u > 0;
+                    if (pair < 4)
+                        net_mma(d + g * 64, a,
+                                ((uint64_t)hi << 32) | (b64 + (pair * UNITS + u) * 64 * 16 / 16),
+                                net_idesc(64), add);
+                    else
+                        net_mma(d + g * 64, a,
+                                ((uint64_t)hi << 32) | (b32 + u * CNN_C * 16 / 16),
+                                net_idesc(CNN_C), add);
                 }
 }
 __device__ __forceinline__ void net_commit(uint64_t *bar) {
@@ -149,17 +173,41 @@ __device__ __forceinline__ void net_tmem_wait(float (&v)[16]) {
                  : "memory");
 }
 
-// Sixteen channels of a row: the sums of the NET_GRP accumulators, in pairs.
-__device__ __forceinline__ void net_sums(float (&v)[16], uint32_t taddr) {
-    float o[16], w[16];
-    net_tmem_load(v, taddr);
-    net_tmem_load(o, taddr + CNN_C);
+// The first row's E1 of every warp of a block, for the last lane of the warp before it (called by
+// the four warps of the block; xch: [3][32] floats of the block, barrier id 1 or 2).
+__device__ __forceinline__ void net_exchange(uint32_t taddr, float *xch, int warp4, int barrier) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float v[16], o[16];
+        net_tmem_load(v, taddr + 32 + h * 16);
+        net_tmem_load(o, taddr + 96 + h * 16);
+        net_tmem_wait(v);
+        net_tmem_wait(o);
+        if (warp4 > 0 && lane == 0)
+#pragma unroll
+            for (int c = 0; c < 16; ++c) xch[(warp4 - 1) * 32 + h * 16 + c] = v[c] + o[c];
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(barrier) : "memory");
+}
+
+// Sixteen channels (half h) of the lane's row: E0 + E1 of the next row.
+__device__ __forceinline__ void net_sums(float (&v)[16], uint32_t taddr, const float *xch,
+                                         int warp4, int h) {
+    const int lane = threadIdx.x & 31;
+    float o[16];
+    net_tmem_load(v, taddr + 32 + h * 16);
+    net_tmem_load(o, taddr + 96 + h * 16);
     net_tmem_wait(v);
     net_tmem_wait(o);
-    net_tmem_load(w, taddr + 2 * CNN_C);
 #pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] += o[c];
-    net_tmem_load(o, taddr + 3 * CNN_C);
+    for (int c = 0; c < 16; ++c) {
+        v[c] = __shfl_down_sync(0xFFFFFFFFu, v[c] + o[c], 1);
+        if (lane == 31) v[c] = warp4 < 3 ? xch[warp4 * 32 + h * 16 + c] : 0.0f;
+    }
+    float w[16];
+    net_tmem_load(w, taddr + h * 16);
+    net_tmem_load(o, taddr + 64 + h * 16);
     net_tmem_wait(w);
     net_tmem_wait(o);
 #pragma unroll
@@ -200,6 +248,7 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
                int cin, int T, int n_tiles, int tiles_per_curve) {
     extern __shared__ __align__(128) unsigned char net_raw[];
     __shared__ uint64_t done[2];  // matrix instructions of row block 0 / 1 complete
+    __shared__ float xch[2][96];
     __shared__ uint32_t s_tmem;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int units1 = net_units(cin);
@@ -210,7 +259,7 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
     float *w4 = reinterpret_cast<float *>(wraw + wsize1 + 2 * net_wbytes(4));  // [co][9]
     float *bias = w4 + CNN_C * CNN_K;                                          // [4][32]
     float *act3 = reinterpret_cast<float *>(net_raw);    // [32][NET_ACT3_LD], after layer 3
-    float *part = act3 + CNN_C * NET_ACT3_LD;            // [4][NET_ROWS]
+    float *part = act3 + CNN_C * NET_ACT3_LD;            // [4][NET_PLD]
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -224,7 +273,7 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
         mbar_init(&done[1], 1);
         fence_mbar_init();
     }
-    // weights: [tap][unit][co][8 ci] (channels past the layer's own are zero)
+    // weights (channels past the layer's own are zero)
     for (int l = 0; l < 3; ++l) {
         const int ci_n = l == 0 ? cin : CNN_C, units = l == 0 ? units1 : 4;
         __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(
@@ -232,8 +281,9 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
         const int n = CNN_K * units * CNN_C * 8;
         for (int i = tid; i < n; i += NET_THREADS) {
             const int e = i & 7, co = (i >> 3) & 31, ku = i >> 8;
-            const int ci = (ku % units) * 8 + e, k = ku / units;
-            dst[i] = ci < ci_n ? net.w[l][(co * ci_n + ci) * CNN_K + k] : __float2bfloat16(0.0f);
+            const int u = ku % units, ci = u * 8 + e, k = ku / units;
+            dst[net_wplace(units, k, u, co, e)] =
+                ci < ci_n ? net.w[l][(co * ci_n + ci) * CNN_K + k] : __float2bfloat16(0.0f);
         }
     }
     for (int i = tid; i < CNN_C * CNN_K; i += NET_THREADS) w4[i] = __bfloat162float(net.w[3][i]);
@@ -295,12 +345,12 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int mb = 0; mb < 2; ++mb) {
                     const uint32_t d = tm + (uint32_t)(mb * NET_GRP * CNN_C);
-                    const uint32_t a_lo = net_desc_lo(x0 + (uint32_t)(mb * 128 * 16), NET_UNIT);
-                    const uint32_t b_lo = net_desc_lo(wl, CNN_C * 16);
+                    const uint32_t a_lo =
+                        net_desc_lo(x0 + (uint32_t)(mb * NET_BLOCK * 16), NET_UNIT);
                     if (units == 2)
-                        net_layer_mma<2>(d, a_lo, b_lo);
+                        net_layer_mma<2>(d, a_lo, wl);
                     else
-                        net_layer_mma<4>(d, a_lo, b_lo);
+                        net_layer_mma<4>(d, a_lo, wl);
                     net_commit(&done[mb]);
                 }
             }
@@ -312,7 +362,7 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
             // epilogue: warps 0-3 the rows of block 0, warps 4-7 of block 1 (in place: the other
             // block's instructions read no row of this one). The last layer's FP32 activations
             // overlay the parts, so it waits for both blocks.
-            const int mb = warp >> 2, r = mb * 128 + (warp & 3) * 32 + lane;
+            const int mb = warp >> 2, warp4 = warp & 3, r = mb * NET_BLOCK + warp4 * 32 + lane;
             bool ok = mbar_wait(&done[mb], phase);
             if (l == 2) {
                 ok = mbar_wait(&done[mb ^ 1], phase) && ok;
@@ -320,13 +370,15 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int t = t0 - 12 + 4 * l + r;
+            const bool mine = warp4 * 32 + lane < NET_BLOCK;  // the block's last lane has no row
             const bool inside = t >= 0 && t < T;
-            const bool own = STORE && inside && t >= t0 && t < t0 + NET_OUT;
+            const bool own = STORE && mine && inside && t >= t0 && t < t0 + NET_OUT;
             const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
+            net_exchange(src, xch[mb], warp4, 1 + mb);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 float v[16];
-                net_sums(v, src + h * 16);
+                net_sums(v, src, xch[mb], warp4, h);
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     const float a = fmaxf(v[c] + bias[l * CNN_C + h * 16 + c], 0.0f);
@@ -336,10 +388,10 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
 #pragma unroll
                     for (int c = 0; c < 16; ++c)
                         net.act[l + 1][((int64_t)b * CNN_C + h * 16 + c) * T + t] = v[c];
-                if (l < 2) {
+                if (l < 2 && mine) {
                     net_store_row(x0 + (uint32_t)(2 * h * NET_UNIT + r * 16), v);
                     net_store_row(x0 + (uint32_t)((2 * h + 1) * NET_UNIT + r * 16), v + 8);
-                } else {
+                } else if (mine) {
 #pragma unroll
                     for (int c = 0; c < 16; ++c) act3[(h * 16 + c) * NET_ACT3_LD + r] = v[c];
                 }
@@ -361,7 +413,7 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
         // layer 4 (one output channel, FP32): 4 bins x 8 input channels per thread
         {
             const int q = tid & 63, cg = tid >> 6;
-            if (q < NET_OUT / 4) {
+            if (q < (NET_OUT + 3) / 4) {
                 float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
@@ -383,13 +435,13 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
                         for (int e = 0; e < 4; ++e) acc[e] = fmaf(wk, xv[e + k], acc[e]);
                     }
                 }
-                *reinterpret_cast<float4 *>(&part[cg * NET_ROWS + 4 * q]) =
+                *reinterpret_cast<float4 *>(&part[cg * NET_PLD + 4 * q]) =
                     make_float4(acc[0], acc[1], acc[2], acc[3]);
             }
             __syncthreads();
             for (int o = tid; o < NET_OUT && t0 + o < T; o += NET_THREADS) {
-                const float z = (part[o] + part[NET_ROWS + o]) +
-                                (part[2 * NET_ROWS + o] + part[3 * NET_ROWS + o]) +
+                const float z = (part[o] + part[NET_PLD + o]) +
+                                (part[2 * NET_PLD + o] + part[3 * NET_PLD + o]) +
                                 bias[3 * CNN_C];
                 if (STORE)
                     net.act[CNN_LAYERS][(int64_t)b * T + t0 + o] = z;
@@ -447,6 +499,7 @@ __global__ void __launch_bounds__(NET_THREADS, 2)
 cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
     extern __shared__ __align__(128) unsigned char net_raw[];
     __shared__ uint64_t done[2];
+    __shared__ float xch[2][96];
     __shared__ uint32_t s_tmem;
     __shared__ double s_loss[NET_THREADS / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -466,13 +519,14 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
         mbar_init(&done[1], 1);
         fence_mbar_init();
     }
-    // flipped, transposed weights of layers 2 and 1: [tap][unit of co][ci][8 co]
+    // flipped, transposed weights of layers 2 and 1 (units of co, rows of ci)
     for (int l = 0; l < 2; ++l) {
         const __nv_bfloat16 *w = l == 0 ? ar.w2 : ar.w1;
         __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(wraw + l * net_wbytes(4));
         for (int i = tid; i < CNN_K * 4 * CNN_C * 8; i += NET_THREADS) {
             const int e = i & 7, ci = (i >> 3) & 31, u = (i >> 8) & 3, k = i >> 10;
-            dst[i] = w[((u * 8 + e) * CNN_C + ci) * CNN_K + (CNN_K - 1 - k)];
+            dst[net_wplace(4, k, u, ci, e)] =
+                w[((u * 8 + e) * CNN_C + ci) * CNN_K + (CNN_K - 1 - k)];
         }
     }
     for (int i = tid; i < CNN_C * CNN_K; i += NET_THREADS) w3[i] = __bfloat162float(ar.w3[i]);
@@ -528,15 +582,16 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int mb = 0; mb < 2; ++mb) {
                     net_layer_mma<4>(tm + (uint32_t)(mb * NET_GRP * CNN_C),
-                                     net_desc_lo(x0 + (uint32_t)(mb * 128 * 16), NET_UNIT),
-                                     net_desc_lo(w0 + (uint32_t)(l * net_wbytes(4)), CNN_C * 16));
+                                     net_desc_lo(x0 + (uint32_t)(mb * NET_BLOCK * 16), NET_UNIT),
+                                     w0 + (uint32_t)(l * net_wbytes(4)));
                     net_commit(&done[mb]);
                 }
             }
             __syncwarp();
-            const int mb = warp >> 2, r = mb * 128 + (warp & 3) * 32 + lane;
+            const int mb = warp >> 2, warp4 = warp & 3, r = mb * NET_BLOCK + warp4 * 32 + lane;
             const int t = t0 - 4 + 4 * l + r;
-            const bool inside = t >= 0 && t < T;
+            const bool mine = warp4 * 32 + lane < NET_BLOCK;  // the block's last lane has no row
+            const bool inside = mine && t >= 0 && t < T;
             const bool own = inside && t >= t0 && t < own_end;
             const int64_t at = (int64_t)b * CNN_C * T + t;
             const float *act = l == 0 ? ar.act2 : ar.act1;
@@ -549,16 +604,17 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
             const bool ok = mbar_wait(&done[mb], phase);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
+            net_exchange(src, xch[mb], warp4, 1 + mb);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 float v[16];
-                net_sums(v, src + h * 16);
+                net_sums(v, src, xch[mb], warp4, h);
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     v[c] = (mask >> (h * 16 + c)) & 1u ? v[c] : 0.0f;
                     if (own) out[at + (int64_t)(h * 16 + c) * T] = v[c];
                 }
-                if (l == 0) {
+                if (l == 0 && mine) {
                     net_store_row(x0 + (uint32_t)(2 * h * NET_UNIT + r * 16), v);
                     net_store_row(x0 + (uint32_t)((2 * h + 1) * NET_UNIT + r * 16), v + 8);
                 }
