@@ -75,3 +75,53 @@ def test_network_tiles(cin, T, B):
     out = torch.empty((B, T), dtype=torch.float32, device="cuda")
     net.forward(torch.from_numpy(f).cuda(), out)
     np.testing.assert_allclose(out.cpu().numpy(), ocnn.probabilities(p, f), rtol=0, atol=2e-5)
+
+
+@pytest.mark.parametrize("n_dur", [2, 3, 7])
+@pytest.mark.parametrize("flat", [False, True])
+def test_fold_shapes(n_dur, flat):
+    """Periods whose phase counts and epochs sit at the edges of the fold's tiles: several duration
+    rows per tile with 1 to 4 rows of lanes at work, the change to whole tiles, ragged last tiles,
+    and winners summed over 1 to 70 epochs. Flat data has equal windows everywhere: the first one
+    wins. Tolerances are the parity tests' (compare_periodic)."""
+    from _parity import compare_periodic
+    from synth.lightcurves import custom
+    step = 120.0 / 86400.0
+    phases = [40, 75, 111, 112, 113, 149, 150, 223, 224, 225, 298, 299, 336, 337, 447, 448, 449, 672,
+              673, 896, 897, 1500, 2699, 2750]
+    periods = np.sort(np.concatenate([np.array(phases) * step, (np.array(phases) - 0.4) * step]))
+    w = custom(seed=n_dur, n_points=2800, cadence_s=120.0,
+               durations_h=np.linspace(0.3, 1.2, n_dur), periods=periods,
+               planets=[] if flat else [dict(P=0.42, t0=0.1, D=0.02, depth=3e-3)])
+    if flat:
+        w.flux[:] = 1.0
+    args = (w.time, w.flux, w.flux_err, w.durations, w.template, periods)
+    kw = dict(cadence=w.cadence, t0_step=w.t0_step)
+    g, o = gpu_search(*args, **kw), oracle_search(*args, **kw)
+    if flat:
+        np.testing.assert_array_equal(g["periodic"]["dlogl"], o["periodic"]["dlogl"])
+        np.testing.assert_array_equal(g["periodic"]["i"], o["periodic"]["i"])
+        np.testing.assert_array_equal(g["periodic"]["j"], o["periodic"]["j"])
+    else:
+        compare_periodic(g, o, periods)
+
+
+@pytest.mark.parametrize("n_points", [40, 300, 5000])
+def test_event_segments(n_points):
+    """Single-transit events whose hidden cells lie in one segment, cross segments and cover the
+    whole grid: the greedy picks of a plain scan over the same linear grid."""
+    from paper_2503_20875_gb300 import Context, cetra_linear_search, cetra_monotransit_search
+    from synth.lightcurves import custom
+    w = custom(seed=n_points, n_points=n_points, cadence_s=120.0, durations_h=(0.4, 1.1, 9.0))
+    ctx = Context(0)
+    grid, depth, _, lr = cetra_linear_search(ctx, w.time, w.flux, w.flux_err, w.durations,
+                                             w.template, cadence=w.cadence, t0_step=w.t0_step)
+    ev = cetra_monotransit_search(ctx, grid, 12)
+    score = np.where(depth > 0, lr, -1.0).astype(np.float64)
+    reach = w.durations / w.t0_step
+    i_all = np.arange(lr.shape[1])
+    for m in range(len(ev["i"])):
+        j, i = np.unravel_index(np.nanargmax(score), score.shape)
+        assert (ev["i"][m], ev["j"][m]) == (i, j)
+        score[:, np.abs(i_all - i) < reach[j]] = -1.0
+    assert len(ev["i"]) == 12 or not np.nanmax(score) > 0
