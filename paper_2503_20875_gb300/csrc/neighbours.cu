@@ -100,23 +100,30 @@ mono_keys_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I, int J, in
     }
 }
 
-// All greedy steps (one block): the best key left becomes the next event (FP64 values from the
-// window's FP32 sums), then the t0 cells within its duration are hidden: |i - i_e| < h =
-// D_j q / (c p) (FP64) -> key 0. Ends early when no key is left.
+// All greedy steps (one block): the best key left becomes the next event, then the t0 cells within
+// its duration are hidden: |i - i_e| < h = D_j q / (c p) (FP64) -> key 0. Ends early when no key
+// is left. The FP64 work (every duration's h before the steps, the events' values from their
+// windows' FP32 sums after them) is a lane each: within a step one lane's divisions were half of
+// its time.
 __global__ void __launch_bounds__(EV_THREADS)
 mono_events_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I,
                    const double *__restrict__ durations, double t_ref, double c, int64_t p,
-                   int64_t q, int64_t n_pad, int shift, int max_events,
+                   int64_t q, int64_t n_pad, int shift, int J, int max_events,
                    unsigned long long *__restrict__ keys,
                    const unsigned long long *__restrict__ top, cetra_event *__restrict__ events,
                    int *__restrict__ n_events) {
     __shared__ unsigned long long seg[EV_SEGMENTS];
     __shared__ unsigned long long red[EV_THREADS / 32];
     __shared__ unsigned long long s_key;
-    __shared__ int64_t s_reach;
+    __shared__ int64_t reach[256];  // integers below h are those below ceil(h)
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     const int n_seg = (int)((I + ((int64_t)1 << shift) - 1) >> shift);
     for (int x = t; x < n_seg; x += EV_THREADS) seg[x] = top[x];
+    if (t < J) {
+        const double span =
+            ceil(__ddiv_rn(__dmul_rn(durations[t], (double)q), __dmul_rn(c, (double)p)));
+        reach[t] = span < (double)I ? (int64_t)span : I;
+    }
     __syncthreads();
     int e = 0;
     for (; e < max_events; ++e) {
@@ -134,28 +141,8 @@ mono_events_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I,
         if (key == 0ull) break;  // uniform
         const int64_t ie = 0xFFFFFF - (int64_t)(key & 0xFFFFFFull);
         const int j = 255 - (int)((key >> 24) & 0xFFull);
-        if (t == 0) {
-            // (one lane: FP64 in all warps would take longer than the rest of the step)
-            // integers below h are those below ceil(h)
-            const double h =
-                __ddiv_rn(__dmul_rn(durations[j], (double)q), __dmul_rn(c, (double)p));
-            const double span = ceil(h);
-            s_reach = span < (double)I ? (int64_t)span : I;
-            const float2 v = ab[(int64_t)j * ld + ie];
-            cetra_event ev;
-            ev.depth = __ddiv_rn((double)v.x, (double)v.y);
-            ev.depth_var = __ddiv_rn(1.0, (double)v.y);
-            ev.dlogl = 0.5 * __dmul_rn((double)v.x, ev.depth);
-            ev.t0 =
-                __dadd_rn(t_ref, __ddiv_rn(__dmul_rn((double)(ie * p - n_pad * q), c), (double)q));
-            ev.duration = durations[j];
-            ev.i = ie;
-            ev.j = j;
-            ev.pad_ = 0;
-            events[e] = ev;
-        }
-        __syncthreads();
-        const int64_t r = s_reach;
+        if (t == 0) events[e].i = (int64_t)key;  // decoded below
+        const int64_t r = reach[j];
         const int64_t lo = max((int64_t)0, ie - r), hi = min(I - 1, ie + r);
         // hide the cells, and work out the maxima of their segments again (32 consecutive cells
         // are of one segment)
@@ -173,6 +160,23 @@ mono_events_kernel(const float2 *__restrict__ ab, int64_t ld, int64_t I,
         __syncthreads();
     }
     if (t == 0) *n_events = e;
+    __syncthreads();
+    for (int x = t; x < e; x += EV_THREADS) {
+        const unsigned long long key = (unsigned long long)events[x].i;
+        const int64_t ie = 0xFFFFFF - (int64_t)(key & 0xFFFFFFull);
+        const int j = 255 - (int)((key >> 24) & 0xFFull);
+        const float2 v = ab[(int64_t)j * ld + ie];
+        cetra_event ev;
+        ev.depth = __ddiv_rn((double)v.x, (double)v.y);
+        ev.depth_var = __ddiv_rn(1.0, (double)v.y);
+        ev.dlogl = 0.5 * __dmul_rn((double)v.x, ev.depth);
+        ev.t0 = __dadd_rn(t_ref, __ddiv_rn(__dmul_rn((double)(ie * p - n_pad * q), c), (double)q));
+        ev.duration = durations[j];
+        ev.i = ie;
+        ev.j = j;
+        ev.pad_ = 0;
+        events[x] = ev;
+    }
 }
 
 unsigned blocks_for(int64_t n, int num_sms) {
@@ -209,7 +213,7 @@ cudaError_t launch_monotransits(cetra_ctx *ctx, const cetra_plan *plan, const fl
     if (e) return e;
     mono_events_kernel<<<1, EV_THREADS, 0, ctx->stream>>>(
         ab, plan->ab_ld, I, plan->d_durations, plan->t_ref, plan->cadence, plan->p, plan->q,
-        plan->n_pad, shift, max_events, keys, top, events, n_events);
+        plan->n_pad, shift, plan->J, max_events, keys, top, events, n_events);
     ctx->launches++;
     return cudaGetLastError();
 }
