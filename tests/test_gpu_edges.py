@@ -125,3 +125,40 @@ def test_event_segments(n_points):
         assert (ev["i"][m], ev["j"][m]) == (i, j)
         score[:, np.abs(i_all - i) < reach[j]] = -1.0
     assert len(ev["i"]) == 12 or not np.nanmax(score) > 0
+
+
+@pytest.mark.parametrize("n_points,max_events", [(2, 1), (40, 1), (5000, 1), (5000, 3)])
+def test_event_scratch_limit(n_points, max_events):
+    """Events in a workspace with one word per t0 cell and event, and nothing past its end
+    written: the first picks of the host form."""
+    import ctypes
+    import torch
+    from paper_2503_20875_gb300 import (Context, Plan, cetra_linear_device, cetra_linear_search,
+                                        cetra_monotransit_search, cetra_monotransits_device,
+                                        cetra_resample_device)
+    from paper_2503_20875_gb300 import _native as N
+    from synth.lightcurves import custom
+    w = custom(seed=n_points, n_points=n_points, cadence_s=120.0, durations_h=(0.4, 1.1, 9.0))
+    ctx = Context(0)
+    grid, _, _, _ = cetra_linear_search(ctx, w.time, w.flux, w.flux_err, w.durations, w.template,
+                                        cadence=w.cadence, t0_step=w.t0_step)
+    ev = cetra_monotransit_search(ctx, grid, max_events)
+    plan = Plan(ctx, w.time, w.flux, w.flux_err, w.durations, w.template, cadence=w.cadence,
+                t0_step=w.t0_step)
+    nb = N.lib.cetra_workspace_bytes(plan.handle, plan.info["n_t0"] + max_events)
+    buf = torch.full((nb + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    ws = buf[:nb]
+    t, f, e = (torch.from_numpy(np.ascontiguousarray(x)).cuda()
+               for x in (w.time, w.flux, w.flux_err))
+    cetra_resample_device(ctx, plan, t, f, e, ws)
+    cetra_linear_device(ctx, plan, ws, None, None, None)
+    rec = ctypes.sizeof(N.cetra_event)
+    d_ev = torch.zeros(max_events * rec, dtype=torch.uint8, device="cuda")
+    d_n = torch.zeros(1, dtype=torch.int32, device="cuda")
+    cetra_monotransits_device(ctx, plan, ws, max_events, d_ev, d_n)
+    torch.cuda.synchronize()
+    raw = d_ev.cpu().numpy().tobytes()
+    got = [N.cetra_event.from_buffer_copy(raw[rec * m:rec * (m + 1)])
+           for m in range(int(d_n.item()))]
+    assert [(x.i, x.j) for x in got] == list(zip(ev["i"], ev["j"]))
+    assert bool((buf[nb:] == 0xA5).all())
