@@ -12,6 +12,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
+#include <new>
 
 #include "internal.h"
 
@@ -216,28 +218,30 @@ int plan_upload(cetra_ctx *ctx, cetra_plan *plan) {
     std::stable_sort(plan->lin_order.begin(), plan->lin_order.end(), [&](int32_t a, int32_t b) {
         return plan->win_padlen[(size_t)a] > plan->win_padlen[(size_t)b];
     });
-    std::vector<unsigned char> host;
-    auto add = [&](const void *src, size_t bytes) {
-        const size_t at = host.size();
-        const unsigned char *b = static_cast<const unsigned char *>(src);
-        host.insert(host.end(), b, b + bytes);
-        host.resize((host.size() + 255) & ~(size_t)255);
+    size_t total = 0;
+    auto place = [&](const auto &v) {
+        const size_t at = total;
+        total += (v.size() * sizeof(v[0]) + 255) & ~(size_t)255;
         return at;
     };
-    auto bytes = [](const auto &v) { return v.size() * sizeof(v[0]); };
-    const size_t o_tab = add(plan->tables.data(), bytes(plan->tables));
-    const size_t o_dur = add(plan->durations.data(), bytes(plan->durations));
-    const size_t o_off = add(plan->win_off.data(), bytes(plan->win_off));
-    const size_t o_a = add(plan->win_a.data(), bytes(plan->win_a));
-    const size_t o_len = add(plan->win_len.data(), bytes(plan->win_len));
-    const size_t o_pad = add(plan->win_padlen.data(), bytes(plan->win_padlen));
-    const size_t o_ord = add(plan->lin_order.data(), bytes(plan->lin_order));
-    cudaError_t e = cudaMalloc(&plan->d_mem, host.size());
+    const size_t o_tab = place(plan->tables), o_dur = place(plan->durations);
+    const size_t o_off = place(plan->win_off), o_a = place(plan->win_a);
+    const size_t o_len = place(plan->win_len), o_pad = place(plan->win_padlen);
+    const size_t o_ord = place(plan->lin_order);
+    std::unique_ptr<unsigned char[]> host(new (std::nothrow) unsigned char[total]);
+    if (!host) return set_error(ctx, CETRA_ENOMEM, "plan upload: host allocation");
+    auto put = [&](const auto &v, size_t at) {
+        std::memcpy(host.get() + at, v.data(), v.size() * sizeof(v[0]));
+    };
+    put(plan->tables, o_tab), put(plan->durations, o_dur), put(plan->win_off, o_off);
+    put(plan->win_a, o_a), put(plan->win_len, o_len), put(plan->win_padlen, o_pad);
+    put(plan->lin_order, o_ord);
+    cudaError_t e = cudaMalloc(&plan->d_mem, total);
     if (e != cudaSuccess) {
         plan->d_mem = nullptr;
         return set_error(ctx, CETRA_ENOMEM, std::string("plan upload: ") + cudaGetErrorString(e));
     }
-    e = cudaMemcpy(plan->d_mem, host.data(), host.size(), cudaMemcpyHostToDevice);
+    e = cudaMemcpy(plan->d_mem, host.get(), total, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return set_error(ctx, CETRA_ECUDA, cudaGetErrorString(e));
     char *base = static_cast<char *>(plan->d_mem);
     plan->d_tables = reinterpret_cast<float2 *>(base + o_tab);
