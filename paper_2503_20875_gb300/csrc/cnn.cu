@@ -40,9 +40,14 @@ constexpr size_t kCombSmemMax = 98 * 1024;  // maps up to 24,576 bins (+ 512 cel
 //
 // Precision: the weights are BF16 values; an FP32 activation is the exact sum of three BF16
 // parts (its leading 8, middle 8 and last 8 bits), so three products with the same weight give
-// the FP32 product exactly. The tensor core's accumulator truncates, so a sum is kept in NET_GRP
-// accumulators (taps 0 and 2, 1 and 3, 4, 6 and 8, 5 and 7; each takes its last and middle parts
-// first), which are added in FP32. Measured error of the probabilities against 64 bits: see cnn_forward.
+// the FP32 product exactly. The tensor core's accumulator truncates, so a sum is kept in four
+// accumulators (net_layer_mma; each takes its last and middle parts first), which are added in
+// FP32. Measured error of the probabilities against 64 bits: 7e-8 (FP32 kernels: 1.1e-7).
+//
+// Measured (256 curves, 16 durations, 4,096 bins): 2,347 us as log1p, four FP32 conv kernels and
+// a sigmoid with every activation in memory, 265 us as this kernel (three parts' products alone:
+// 76 us at the measured BF16 rate). Bound: the instructions' reads of the activations and the
+// epilogues (splitting the next layer's input), in turn between the two blocks of an SM.
 //
 // Halo: layer l's row r is bin t0 - 16 + 4 l + r. A tile computes NET_ROWS = 254 rows of the
 // first three layers in place (rows past the last valid one are never used): 254, 246, 238
@@ -112,7 +117,7 @@ __device__ __forceinline__ void net_mma(uint32_t d, uint64_t a, uint64_t b, uint
 // Reading the activations is the bound, so an instruction takes two taps: N = 64 are the 32
 // output channels of taps 2 p and 2 p + 1, both on the rows of tap 2 p, and the second tap's sums
 // belong one row further down: out[r] = E0[r] + E1[r + 1] (net_sums). A block of 128 rows
-// therefore completes 127. One tap per instruction: 291 us for 256 curves x 16 durations.
+// therefore completes 127. 256 curves x 16 durations: 265 us; one tap per instruction: 291 us.
 // Accumulators: E0 and E1 of pairs 0-1 and of pairs 2-4 (columns 0, 32, 64, 96), four partial
 // sums of every output. Consecutive instructions go to different ones, and every offset is a
 // constant of the unrolled code (worked out in a loop, one accumulator after the other, the
@@ -478,8 +483,9 @@ __device__ __forceinline__ float bce_loss(float z, float y, float wpos) {
 // pass run in reverse: G_3 (one channel) -> G_2 in FP32, G_2 -> G_1 -> G_0 as matrix
 // instructions, each masked where the layer's activation is not positive (ReLU). Rows: G_2's
 // row i is bin t0 - 8 + i, G_1's row r bin t0 - 4 + r, G_0's row r bin t0 + r.
-// Measured with the weight gradients below (32 curves, 16 durations): 940 us a step when each
-// layer was a transpose, an FP32 conv and a mask kernel and the weight gradients met in atomics.
+// Measured (32 curves, 16 durations): a training step took 940 us when each layer's gradient was a
+// transpose, an FP32 conv and a mask kernel and the weight gradients met in atomics (the forward
+// pass fused already); with this kernel (46 us) and the weight gradients below (152 us), 304 us.
 constexpr int BACK_OUT = NET_ROWS - 8;
 constexpr int BACK_G4 = NET_XROWS + 8;  // bins of G_3 a tile needs
 inline size_t back_smem() {
@@ -961,8 +967,8 @@ __global__ void cnn_map_kernel(const float *__restrict__ prob, const float *__re
 // block per (interval, curve) doing it that was two thirds of the time. A curve's map is staged in
 // shared memory when it fits; the trials' own FP64 arithmetic (Pb, F, phase count) is done once
 // per trial into shared memory, COMB_CHUNK trials at a time.
-// Measured (256 curves, 4,096 bins, 512 intervals): 15.8 ms with a block per (interval, curve)
-// and a lane per (trial, phase).
+// Measured (256 curves, 4,096 bins, 512 intervals): 5.3 ms; 15.8 ms with a block per (interval,
+// curve) and a lane per (trial, phase). The shared loads alone: 2.2 ms.
 constexpr int COMB_CHUNK = 256;
 constexpr int COMB_ROWS = 16;
 constexpr int COMB_THREADS = 256;
@@ -971,7 +977,7 @@ constexpr int COMB_THREADS = 256;
 // trial. Phases of equal epoch counts are compared by their sums (a rounded division by the same
 // number keeps their order), and the square root and the division are taken only where they may
 // beat `best`: m / sqrt(n) > best needs m^2 > best^2 n (1 - 2^-17), whose left side and right
-// side are rounded by far less. PAD: cells up to 32 R past the last valid one may be read (a
+// side are rounded by far less (below 1e-15 the squares might not be normal). PAD: cells up to 32 R past the last valid one may be read (a
 // phase that has no further epoch is done with, so what is added to it does not matter).
 // Short trials (nph <= 16, R = 1) share a warp: `mine` is the lane's phase and F its own trial's.
 template <int R, bool PAD>
@@ -1010,7 +1016,7 @@ __device__ __forceinline__ float comb_unit(const float *__restrict__ src, uint32
         for (int r = 0; r < R; ++r)
             if (mine + 32 * r >= lim && mine + 32 * r < have) m = fmaxf(m, s[r]);
         const float fn = (float)n;
-        if (m > 0.0f && !(m * m < best * best * fn * (1.0f - 1.0f / 131072.0f)))
+        if (m > 0.0f && !(best > 1e-15f && m * m < best * best * fn * (1.0f - 1.0f / 131072.0f)))
             best = fmaxf(best, m / sqrtf(fn));
         if (lim <= ph0) return best;
 #pragma unroll
