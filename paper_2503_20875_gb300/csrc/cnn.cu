@@ -485,7 +485,7 @@ __device__ __forceinline__ float bce_loss(float z, float y, float wpos) {
 // row i is bin t0 - 8 + i, G_1's row r bin t0 - 4 + r, G_0's row r bin t0 + r.
 // Measured (32 curves, 16 durations): a training step took 940 us when each layer's gradient was a
 // transpose, an FP32 conv and a mask kernel and the weight gradients met in atomics (the forward
-// pass fused already); with this kernel (46 us) and the weight gradients below (152 us), 304 us.
+// pass fused already); with this kernel (44 us) and the weight gradients below (152 us), 302 us.
 constexpr int BACK_OUT = NET_ROWS - 8;
 constexpr int BACK_G4 = NET_XROWS + 8;  // bins of G_3 a tile needs
 inline size_t back_smem() {

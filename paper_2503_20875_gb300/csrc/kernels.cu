@@ -281,7 +281,7 @@ linear_kernel(const float2 *__restrict__ grid, int64_t n_grid,
 //
 // A winner's sum is a chain of dependent FP64 adds behind loads whose addresses take FP64
 // arithmetic too; with a thread per period the longest chain (one term per epoch) was the
-// kernel's time whatever the number of periods (38 us at 2,000 periods and 54 epochs; now 6 us). FIN_LANES
+// kernel's time whatever the number of periods (38 us at 2,000 periods and 54 epochs; 11 us now). FIN_LANES
 // neighbouring lanes now share a winner, each with FIN_CHAINS sums in flight: chain m of lane l
 // adds epochs l + FIN_LANES m, + FIN_LANES FIN_CHAINS, ..., and the chains' and lanes' sums are
 // added in pairs (every caller the same way, so that equal models stay equal). More lanes would
