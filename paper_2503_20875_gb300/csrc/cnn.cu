@@ -977,8 +977,9 @@ constexpr int COMB_THREADS = 256;
 // trial. Phases of equal epoch counts are compared by their sums (a rounded division by the same
 // number keeps their order), and the square root and the division are taken only where they may
 // beat `best`: m / sqrt(n) > best needs m^2 > best^2 n (1 - 2^-17), whose left side and right
-// side are rounded by far less (below 1e-15 the squares might not be normal). PAD: cells up to 32 R past the last valid one may be read (a
-// phase that has no further epoch is done with, so what is added to it does not matter).
+// side are rounded by far less (below 1e-15 the squares might not be normal). PAD: cells up to
+// 32 R past the last valid one may be read (a phase that has no further epoch is done with, so
+// what is added to it does not matter).
 // Short trials (nph <= 16, R = 1) share a warp: `mine` is the lane's phase and F its own trial's.
 template <int R, bool PAD>
 __device__ __forceinline__ float comb_unit(const float *__restrict__ src, uint32_t V,
