@@ -331,10 +331,11 @@ __device__ __forceinline__ void offer_best(fold_smem &sm, int g, float lr2, uint
 }
 
 // The better of a lane's best window (lr2, at) and the window sum (x, y) at index here, which
-// comes later in flat order: 2 LR = x * (x / y); a null sum gives NaN, never a maximum.
+// comes later in flat order: 2 LR = x * (x / y). A null sum (y = 0) is never a maximum: x is not
+// zero with it where a template value's square underflows, and the quotient would be infinite.
 __device__ __forceinline__ void take_max(float x, float y, uint32_t here, float &lr2,
                                          uint32_t &at) {
-    const float v = x * __fdividef(x, y);
+    const float v = y > 0.0f ? x * __fdividef(x, y) : -1.0f;
     if (v > lr2) {
         lr2 = v;
         at = here;

@@ -162,3 +162,29 @@ def test_event_scratch_limit(n_points, max_events):
            for m in range(int(d_n.item()))]
     assert [(x.i, x.j) for x in got] == list(zip(ev["i"], ev["j"]))
     assert bool((buf[nb:] == 0xA5).all())
+
+
+@pytest.mark.parametrize("n_points,n_dur,n_per,steps", [
+    (300, 1, 12, (310, 440)),      # epoch slices
+    (2000, 1, 12, (2010, 2600)),   # whole tiles
+    (20, 4, 4900, (29, 60)),       # several durations per tile
+])
+def test_null_sum_is_never_a_maximum(n_points, n_dur, n_per, steps):
+    """A template whose ends are so small that their squares underflow (m = 1e-23): a window that
+    meets the data with such a sample alone has B = 0 and A not 0, and a phase with only such
+    windows is null. Periods longer than the curve make it a phase of its own. The winners are
+    those of the 64-bit search, in which the end samples weigh nothing."""
+    from _parity import compare_periodic
+    from synth.lightcurves import custom
+    c = 120.0 / 86400.0
+    periods = np.linspace(steps[0], steps[1], n_per) * c
+    w = custom(seed=n_points, n_points=n_points, cadence_s=120.0,
+               planets=[dict(P=1e3, t0=0.5 * n_points * c, D=9.0 * c, depth=2e-2)])
+    d = np.array([2.0, 4.0, 6.0, 8.0])[4 - n_dur:] * c
+    tmpl = np.ones(1024, np.float32)
+    tmpl[0] = tmpl[-1] = 1e-23
+    args = (w.time, w.flux, w.flux_err, d, tmpl, periods)
+    kw = dict(cadence=c, t0_step=c)
+    g, o = gpu_search(*args, **kw), oracle_search(*args, **kw)
+    assert np.isnan(g["dlogl"][-1, -1]) and np.isfinite(o["dlogl"][-1, -1])  # B = 0, A not 0
+    compare_periodic(g, o, periods)
