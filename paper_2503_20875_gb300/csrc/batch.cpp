@@ -571,7 +571,9 @@ int cetra_batch_search_proposed(cetra_ctx *ctx, cetra_batch *b, cetra_cnn *cnn, 
         bw[(size_t)c] = (double)width * b->plan->t0_step;
         nv[(size_t)c] = (int)((I + width - 1) / width);
     }
-    const size_t nf = (size_t)n * J * T, nm = (size_t)n * T, ns = (size_t)n * n_intervals;
+    // (the FP64 bin widths follow the scores: an even number of those)
+    const size_t nf = (size_t)n * J * T, nm = (size_t)n * T;
+    const size_t ns = ((size_t)n * n_intervals + 1) & ~(size_t)1;
     char *mem = nullptr;
     const size_t bytes = (nf + 2 * nm + ns) * sizeof(float) + (size_t)n * (sizeof(double) + sizeof(int)) + 1024;
     device_guard dguard(ctx->device);

@@ -381,3 +381,22 @@ def test_learned_proposal_gain():
     assert res["learned"][0] >= res["untrained"][0] + 0.05 * n
     assert res["learned"][0] >= res["random"][0] + 0.2 * n
     assert res["learned"][0] >= 0.75 * n_full
+
+
+def test_search_proposed_with_an_odd_number_of_scores():
+    """Odd curves x odd intervals: the scores of the one-call form end on an odd float, and the
+    FP64 bin widths placed after them have to stay aligned. The same models and fold work as the
+    step by step proposal."""
+    from paper_2503_20875_gb300 import CNN, proposal
+    ctx, b, _ = _batch(3, seed=35, max_sectors=2, ratio=None)
+    net = CNN(ctx, b.info["n_dur"], n_bins=512, max_batch=2, seed=6)
+    geo = proposal.geometry(b)
+    p_hi = proposal.period_max(geo)
+    one, n_it1, n_per1 = b.search_proposed(net, n_intervals=101, p_lo=0.5, p_hi=p_hi,
+                                           top_frac=0.1)
+    m = proposal.learned_map(ctx, net, b.features(512))
+    steps, n_it2, n_per2 = proposal.propose_and_fold(ctx, b, m, p_hi, 0.1, n_intervals=101,
+                                                     geo=geo)
+    assert (n_it1, n_per1) == (n_it2, n_per2)
+    for key in ("k", "i", "j", "dlogl", "period", "t0"):
+        np.testing.assert_array_equal(one[key], steps[key])
