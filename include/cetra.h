@@ -436,8 +436,9 @@ int cetra_cnn_get_params(cetra_ctx *ctx, const cetra_cnn *cnn, float *host_param
  * state (moments and step count). Blocks. */
 int cetra_cnn_set_params(cetra_ctx *ctx, cetra_cnn *cnn, const float *host_params);
 /* Probabilities for B <= max_batch curves: d_features device FP32 [B][in][n_bins] (read only),
- * d_prob device FP32 [B][n_bins] (written), both caller-owned. Asynchronous on the context's
- * stream. Errors: CETRA_EINVAL (NULL pointers, B outside 1..max_batch), CETRA_ECUDA. */
+ * d_prob device FP32 [B][n_bins] (written), both caller-owned; they may overlap (the features
+ * are overwritten there once they are used). Asynchronous on the context's stream.
+ * Errors: CETRA_EINVAL (NULL pointers, B outside 1..max_batch), CETRA_ECUDA. */
 int cetra_cnn_forward(cetra_ctx *ctx, cetra_cnn *cnn, const float *d_features, int B,
                       float *d_prob);
 /* Forward + backward of the weighted binary cross-entropy with logits against d_labels

@@ -1330,7 +1330,17 @@ int cetra_cnn_forward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features, int
         return set_error(ctx, CETRA_EINVAL, "cnn_forward: bad argument");
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
-    if (!e) e = forward(ctx, n, d_features, B, d_prob);
+    // One kernel reads the features (a halo of 16 bins per tile too) and writes the probabilities:
+    // where the two overlap, these go to the network's own buffer first.
+    const size_t rows = (size_t)B * n->T;
+    const uintptr_t f0 = reinterpret_cast<uintptr_t>(d_features);
+    const uintptr_t p0 = reinterpret_cast<uintptr_t>(d_prob);
+    const bool overlap = p0 < f0 + rows * n->cin * sizeof(float) && f0 < p0 + rows * sizeof(float);
+    float *prob = overlap ? n->d_act[CNN_LAYERS] : d_prob;
+    if (!e) e = forward(ctx, n, d_features, B, prob);
+    if (!e && overlap)
+        e = cudaMemcpyAsync(d_prob, prob, rows * sizeof(float), cudaMemcpyDeviceToDevice,
+                            ctx->stream);
     return e ? cnn_fail(ctx, e, "cnn_forward") : CETRA_OK;
 }
 

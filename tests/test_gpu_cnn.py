@@ -400,3 +400,22 @@ def test_search_proposed_with_an_odd_number_of_scores():
     assert (n_it1, n_per1) == (n_it2, n_per2)
     for key in ("k", "i", "j", "dlogl", "period", "t0"):
         np.testing.assert_array_equal(one[key], steps[key])
+
+
+@pytest.mark.parametrize("cin,T,B,shift", [(1, 1024, 5, 0), (4, 768, 3, 0), (4, 768, 3, 2000),
+                                           (3, 512, 2, -300)])
+def test_forward_into_the_features(cin, T, B, shift):
+    """Probabilities written over the features they come from (in place, further on, and from
+    before the features): the same bits as into a buffer of their own."""
+    torch = _torch()
+    ctx, net, _ = _net(cin, T, B, seed=40 + cin)
+    f, _ = _inputs(B, cin, T, seed=5)
+    pad = 512
+    buf = torch.zeros(pad + f.size + B * T, dtype=torch.float32, device="cuda")
+    feats = buf[pad:pad + f.size].view(B, cin, T)
+    feats.copy_(torch.from_numpy(f))
+    own = torch.empty((B, T), dtype=torch.float32, device="cuda")
+    net.forward(feats, own)
+    over = buf[pad + shift:pad + shift + B * T].view(B, T)
+    net.forward(feats, over)
+    assert torch.equal(over, own)
