@@ -437,7 +437,8 @@ int cetra_cnn_get_params(cetra_ctx *ctx, const cetra_cnn *cnn, float *host_param
 int cetra_cnn_set_params(cetra_ctx *ctx, cetra_cnn *cnn, const float *host_params);
 /* Probabilities for B <= max_batch curves: d_features device FP32 [B][in][n_bins] (read only),
  * d_prob device FP32 [B][n_bins] (written), both caller-owned; they may overlap (the features
- * are overwritten there once they are used). Asynchronous on the context's stream.
+ * are overwritten there once they are used). Asynchronous on the context's stream; where a
+ * bounded device wait gave up, probabilities are NaN and cetra_cnn_status says so.
  * Errors: CETRA_EINVAL (NULL pointers, B outside 1..max_batch), CETRA_ECUDA. */
 int cetra_cnn_forward(cetra_ctx *ctx, cetra_cnn *cnn, const float *d_features, int B,
                       float *d_prob);
@@ -445,12 +446,26 @@ int cetra_cnn_forward(cetra_ctx *ctx, cetra_cnn *cnn, const float *d_features, i
  * (device FP32 [B][n_bins], 0 or 1), mean over bins, positive weight pos_weight. Leaves the
  * gradient on the device for cetra_cnn_adam; *loss and host_grads (flat, like the
  * parameters) are filled when not NULL (that synchronises). Weight gradients are summed with
- * atomics, so their last bits may differ from run to run. Errors as cetra_cnn_forward. */
+ * atomics, so their last bits may differ from run to run. Where a bounded device wait gave up,
+ * loss and gradient are NaN and cetra_cnn_status says so.
+ * Errors as cetra_cnn_forward, and CETRA_ETIMEOUT when it synchronised and a wait gave up. */
 int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *cnn, const float *d_features,
                        const float *d_labels, int B, float pos_weight, double *loss,
                        float *host_grads);
+/* Status word of a network: 0, or CETRA_ETIMEOUT if a bounded device wait of its kernels gave up
+ * since the word was last read or the last cetra_cnn_backward or cetra_batch_search_proposed
+ * began (these clear it, and report it themselves when they synchronise). Reading it clears it.
+ * Synchronises the context's stream. Errors: CETRA_EINVAL (NULL argument), CETRA_ECUDA. */
+int cetra_cnn_status(cetra_ctx *ctx, cetra_cnn *cnn, int *status);
+/* Self-test of the network's bounded waits: until the next such call, the tensor-core work of
+ * one tile of the forward pass and one of the gradient pass (index over all curves' tiles;
+ * negative: none) is left out, and a wait gives up after wait_cycles SM clocks (0: the normal
+ * limit, about a second). Errors: CETRA_EINVAL (NULL cnn, wait_cycles < 0). */
+int cetra_selftest_cnn_waits(cetra_cnn *cnn, int forward_tile, int gradient_tile,
+                             int64_t wait_cycles);
 /* One bias-corrected Adam step with the last gradient on the FP32 parameters, then the BF16
- * weights are re-rounded. Asynchronous. */
+ * weights are re-rounded. Asynchronous. Parameters and moments stay as they are when a wait of
+ * that gradient's kernels gave up. */
 int cetra_cnn_adam(cetra_ctx *ctx, cetra_cnn *cnn, float lr, float beta1, float beta2,
                    float eps);
 /* Proposal map d_map[b][t] = d_prob[b][t] * max_j max(d_features[b][j][t], 0): the network's

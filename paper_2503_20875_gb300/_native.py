@@ -139,6 +139,8 @@ SIGNATURES = {
     "cetra_cnn_forward": (_INT, [_P, _P, _P, _INT, _P]),
     "cetra_cnn_backward": (_INT, [_P, _P, _P, _P, _INT, ctypes.c_float,
                                   ctypes.POINTER(ctypes.c_double), _P]),
+    "cetra_cnn_status": (_INT, [_P, _P, ctypes.POINTER(_INT)]),
+    "cetra_selftest_cnn_waits": (_INT, [_P, _INT, _INT, _I64]),
     "cetra_cnn_adam": (_INT, [_P, _P, ctypes.c_float, ctypes.c_float, ctypes.c_float,
                               ctypes.c_float]),
     "cetra_batch_run_proposed": (_INT, [_P, _P, _P, _INT, ctypes.c_double, ctypes.c_double,

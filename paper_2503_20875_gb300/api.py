@@ -600,6 +600,18 @@ class CNN:
               self.ctx.handle, "cnn_backward")
         return (loss.value, g) if grads else loss.value
 
+    def status(self):
+        """0, or CETRA_ETIMEOUT if a device wait gave up since the last look (which clears it)."""
+        v = ctypes.c_int(0)
+        check(N.lib.cetra_cnn_status(self.ctx.handle, self.handle, ctypes.byref(v)),
+              self.ctx.handle, "cnn_status")
+        return v.value
+
+    def selftest_waits(self, forward_tile=-1, gradient_tile=-1, wait_cycles=0):
+        """Leave one tile's tensor-core work out, so that the waits for it run out."""
+        check(N.lib.cetra_selftest_cnn_waits(self.handle, int(forward_tile), int(gradient_tile),
+                                             int(wait_cycles)))
+
     def adam(self, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8):
         check(N.lib.cetra_cnn_adam(self.ctx.handle, self.handle, float(lr), float(beta1),
                                    float(beta2), float(eps)), self.ctx.handle, "cnn_adam")

@@ -587,6 +587,8 @@ int cetra_batch_search_proposed(cetra_ctx *ctx, cetra_batch *b, cetra_cnn *cnn, 
     int rc = CETRA_OK;
     if (!e) e = cudaMemcpyAsync(d_bw, bw.data(), (size_t)n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream);
     if (!e) e = cudaMemcpyAsync(d_nv, nv.data(), (size_t)n * sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
+    int *status = cnn_status_word(cnn);
+    if (!e) e = cudaMemsetAsync(status, 0, sizeof(int), ctx->stream);
     if (e) rc = cuda_fail(ctx, e, "batch_search_proposed");
     if (rc == CETRA_OK) rc = cetra_batch_features(ctx, b, T, feat);
     for (int a = 0; rc == CETRA_OK && a < n; a += mb)
@@ -598,8 +600,15 @@ int cetra_batch_search_proposed(cetra_ctx *ctx, cetra_batch *b, cetra_cnn *cnn, 
     if (rc == CETRA_OK)
         rc = cetra_batch_run_proposed(ctx, b, scores, n_intervals, p_lo, p_hi, top_frac, 0, best,
                                       n_items_out, n_periods_out, nullptr);
-    cudaStreamSynchronize(ctx->stream);
+    int timed_out = 0;  // of the network's waits
+    if (rc == CETRA_OK)
+        e = cudaMemcpyAsync(&timed_out, status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream);
+    const cudaError_t es = cudaStreamSynchronize(ctx->stream);
     cudaFree(mem);
+    if (rc == CETRA_OK && (e || es))
+        rc = cuda_fail(ctx, e ? e : es, "batch_search_proposed");
+    if (rc == CETRA_OK && timed_out)
+        rc = set_error(ctx, CETRA_ETIMEOUT, "batch_search_proposed: a device wait timed out");
     return rc;
 }
 

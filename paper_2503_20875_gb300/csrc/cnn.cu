@@ -85,10 +85,28 @@ __device__ __forceinline__ int net_wplace(int units, int k, int u, int co, int e
                  : (4 * units * 64 + u * CNN_C + co) * 8 + e;
 }
 
+// Words of a network on the device that its kernels leave beside their outputs.
+struct net_words {
+    double loss;
+    int next[CNN_LAYERS];  // tiles of the weight gradients handed out
+    int status;            // 0, or CETRA_ETIMEOUT: a bounded wait gave up
+    int lost;              // not 0: a wait of the last gradient's launches gave up
+};
+
+// Bounded waits of a launch: a wait gives up after `limit` SM clocks, is recorded in the status
+// word, and the block's remaining outputs are NaN. The self-test leaves the matrix instructions
+// of tile `skip` out (-1: none), so that the waits for them run out.
+struct net_waits {
+    int *status;
+    long long limit;
+    int skip;
+};
+
 struct net_layers {
     const __nv_bfloat16 *w[CNN_LAYERS];  // [co][ci][9], BF16
     const float *bias[CNN_LAYERS];
     float *act[CNN_LAYERS + 1];          // training: log1p(features), the activations, the logits
+    net_waits wait;
 };
 
 // Matrix descriptor of a K-major operand without swizzle: rows 16 bytes apart, 8-row groups 128
@@ -346,7 +364,7 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
         for (int l = 0; l < 3; ++l) {
             const int units = l == 0 ? units1 : 4;
             const uint32_t wl = w0 + (l == 0 ? 0 : wsize1 + (l - 1) * net_wbytes(4));
-            if (tid == 0) {
+            if (tid == 0 && tile != net.wait.skip) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int mb = 0; mb < 2; ++mb) {
                     const uint32_t d = tm + (uint32_t)(mb * NET_GRP * CNN_C);
@@ -368,9 +386,9 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
             // block's instructions read no row of this one). The last layer's FP32 activations
             // overlay the parts, so it waits for both blocks.
             const int mb = warp >> 2, warp4 = warp & 3, r = mb * NET_BLOCK + warp4 * 32 + lane;
-            bool ok = mbar_wait(&done[mb], phase);
+            bool ok = mbar_wait(&done[mb], phase, net.wait.limit);
             if (l == 2) {
-                ok = mbar_wait(&done[mb ^ 1], phase) && ok;
+                ok = mbar_wait(&done[mb ^ 1], phase, net.wait.limit) && ok;
                 __syncthreads();
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -404,15 +422,20 @@ cnn_net_kernel(const float *__restrict__ features, net_layers net, float *__rest
             phase ^= 1u;
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             fence_proxy_async();
-            failed = __syncthreads_or(!ok);  // a wait gave up: the tile's outputs are NaN
+            failed = __syncthreads_or(!ok);
             if (failed) break;
         }
-        if (failed) {
-            mbar_wait(&done[0], phase ^ 1u);  // (bounded) before the tensor memory goes
-            mbar_wait(&done[1], phase ^ 1u);
+        if (failed) {  // a wait gave up: this and the block's later tiles are NaN
+            if (tid == 0) atomicExch(net.wait.status, CETRA_ETIMEOUT);
+            mbar_wait(&done[0], phase ^ 1u, net.wait.limit);  // before the tensor memory goes
+            mbar_wait(&done[1], phase ^ 1u, net.wait.limit);
             float *out = STORE ? net.act[CNN_LAYERS] : prob;
-            for (int o = tid; o < NET_OUT && t0 + o < T; o += NET_THREADS)
-                out[(int64_t)b * T + t0 + o] = __int_as_float(0x7fc00000);
+            for (; tile < n_tiles; tile += gridDim.x) {
+                const int bb = tile / tiles_per_curve;
+                const int at = (tile - bb * tiles_per_curve) * NET_OUT;
+                for (int o = tid; o < NET_OUT && at + o < T; o += NET_THREADS)
+                    out[(int64_t)bb * T + at + o] = __int_as_float(0x7fc00000);
+            }
             break;
         }
         // layer 4 (one output channel, FP32): 4 bins x 8 input channels per thread
@@ -499,6 +522,7 @@ struct back_args {
     double *loss;
     float wpos;
     int64_t n;                               // bins of the batch
+    net_waits wait;
 };
 
 __global__ void __launch_bounds__(NET_THREADS, 2)
@@ -584,7 +608,7 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
         fence_proxy_async();
         __syncthreads();
         for (int l = 0; l < 2; ++l) {
-            if (tid == 0) {
+            if (tid == 0 && tile != ar.wait.skip) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 for (int mb = 0; mb < 2; ++mb) {
                     net_layer_mma<4>(tm + (uint32_t)(mb * NET_GRP * CNN_C),
@@ -607,7 +631,7 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
 #pragma unroll
                 for (int c = 0; c < CNN_C; ++c)
                     mask |= (act[at + (int64_t)c * T] > 0.0f ? 1u : 0u) << c;
-            const bool ok = mbar_wait(&done[mb], phase);
+            const bool ok = mbar_wait(&done[mb], phase, ar.wait.limit);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t src = tm + (uint32_t)(mb * NET_GRP * CNN_C) + ((uint32_t)(warp & 3) << 21);
             net_exchange(src, xch[mb], warp4, 1 + mb);
@@ -631,9 +655,10 @@ cnn_back_kernel(back_args ar, int T, int n_tiles, int tiles_per_curve) {
             failed = __syncthreads_or(!ok);
             if (failed) break;
         }
-        if (failed) {  // a wait gave up: the loss says so
-            mbar_wait(&done[0], phase ^ 1u);  // (bounded) before the tensor memory goes
-            mbar_wait(&done[1], phase ^ 1u);
+        if (failed) {  // a wait gave up: the loss is NaN, and the gradient by the status word
+            if (tid == 0) atomicExch(ar.wait.status, CETRA_ETIMEOUT);
+            mbar_wait(&done[0], phase ^ 1u, ar.wait.limit);  // before the tensor memory goes
+            mbar_wait(&done[1], phase ^ 1u, ar.wait.limit);
             loss = __longlong_as_double(0x7ff8000000000000ll);
             break;
         }
@@ -676,6 +701,8 @@ struct wgrad_args {
     wgrad_job job[CNN_LAYERS];
     const float *logits, *labels;  // [B][T]
     int *next;                     // [layer] tiles handed out beyond each block's first (zeroed)
+    const int *status;             // not 0: a wait gave up, the gradient is NaN
+    int *lost;                     // the status word at the time of the gradient
     float wpos;
     int64_t n;
     int B, T;
@@ -907,7 +934,9 @@ cnn_grad_sum_kernel(wgrad_args ar, float *__restrict__ grads) {
         for (int r = 1; r < GS_ROWS; ++r) sum += red[r][lane];
         int64_t off = 0;
         for (int l = 0; l < (int)blockIdx.y; ++l) off += ar.job[l].size;
-        grads[off + i] = sum;
+        const int status = *ar.status;
+        grads[off + i] = status == 0 ? sum : __int_as_float(0x7fc00000);
+        if (i == 0 && blockIdx.y == 0) *ar.lost = status;
     }
 }
 
@@ -917,12 +946,13 @@ __global__ void cnn_round_kernel(const float *__restrict__ w, __nv_bfloat16 *__r
     if (i < n) wb[i] = __float2bfloat16_rn(w[i]);
 }
 
-// Adam on the FP32 training copy.
+// Adam on the FP32 training copy. Nothing changes when a wait of the gradient's launches gave up.
 __global__ void cnn_adam_kernel(float *__restrict__ w, const float *__restrict__ g,
                                 float *__restrict__ m, float *__restrict__ v, int64_t n, float lr,
-                                float b1, float b2, float eps, float c1, float c2) {
+                                float b1, float b2, float eps, float c1, float c2,
+                                const int *__restrict__ lost) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *lost != 0) return;
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
@@ -1150,9 +1180,11 @@ struct cetra_cnn {
     float *d_act[CNN_LAYERS + 1] = {};  // act[0] = log1p(features), act[l + 1] = layer l output
     float *d_g[CNN_LAYERS - 1] = {};  // gradients of layers 0 .. 2 [max_batch][32][T]
     float *d_part = nullptr;          // partial weight gradients of the blocks
-    double *d_loss = nullptr;
+    net_words *d_words = nullptr;
     void *d_mem = nullptr;
     int adam_step = 0;
+    long long wait_limit = FT_WAIT_CYCLES;
+    int skip[2] = {-1, -1};  // self-test: tiles of the forward and the gradient pass left out
 };
 
 namespace {
@@ -1174,6 +1206,7 @@ cudaError_t forward(cetra_ctx *ctx, cetra_cnn *n, const float *features, int B, 
         net.bias[l] = n->d_params + n->b_off[l];
     }
     for (int l = 0; l <= CNN_LAYERS; ++l) net.act[l] = n->d_act[l];
+    net.wait = {&n->d_words->status, n->wait_limit, n->skip[0]};
     const int per = (n->T + NET_OUT - 1) / NET_OUT;
     const int64_t tiles = (int64_t)per * B;
     if (tiles > 2147483647) return cudaErrorInvalidConfiguration;
@@ -1193,6 +1226,8 @@ cudaError_t round_weights(cetra_ctx *ctx, cetra_cnn *n) {
 }
 
 }  // namespace
+
+int *cnn_status_word(cetra_cnn *n) { return &n->d_words->status; }
 
 extern "C" {
 
@@ -1253,7 +1288,7 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
     n->d_m = reinterpret_cast<float *>(take(P * 4));
     n->d_v = reinterpret_cast<float *>(take(P * 4));
     n->d_wb = reinterpret_cast<__nv_bfloat16 *>(take(P * 2));
-    n->d_loss = reinterpret_cast<double *>(take(8 + CNN_LAYERS * sizeof(int)));
+    n->d_words = reinterpret_cast<net_words *>(take(sizeof(net_words)));
     for (int l = 0; l < CNN_LAYERS; ++l) n->d_act[l] = reinterpret_cast<float *>(take(act * 4));
     n->d_act[CNN_LAYERS] = reinterpret_cast<float *>(take(logits * 4));
     for (float *&g : n->d_g) g = reinterpret_cast<float *>(take(act * 4));
@@ -1261,6 +1296,7 @@ int cetra_cnn_create(cetra_ctx *ctx, int in_channels, int n_bins, int max_batch,
     e = cudaMemcpy(n->d_params, init.data(), P * 4, cudaMemcpyHostToDevice);
     if (!e) e = cudaMemset(n->d_m, 0, P * 4);
     if (!e) e = cudaMemset(n->d_v, 0, P * 4);
+    if (!e) e = cudaMemset(n->d_words, 0, sizeof(net_words));
     for (auto fn : {cnn_net_kernel<false>, cnn_net_kernel<true>})
         if (!e)
             e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1352,9 +1388,8 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
     const int T = n->T;
     device_guard dguard(ctx->device);
     cudaError_t e = dguard.status;
+    if (!e) e = cudaMemsetAsync(n->d_words, 0, sizeof(net_words), ctx->stream);
     if (!e) e = forward(ctx, n, d_features, B, nullptr);
-    // the loss and the tile counters behind it
-    if (!e) e = cudaMemsetAsync(n->d_loss, 0, 8 + CNN_LAYERS * sizeof(int), ctx->stream);
     if (!e) {
         back_args ar{};
         ar.w1 = n->d_wb + n->w_off[1];
@@ -1368,7 +1403,8 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
         ar.g0 = n->d_g[0];
         ar.g1 = n->d_g[1];
         ar.g2 = n->d_g[2];
-        ar.loss = n->d_loss;
+        ar.loss = &n->d_words->loss;
+        ar.wait = {&n->d_words->status, n->wait_limit, n->skip[1]};
         ar.wpos = pos_weight;
         ar.n = (int64_t)B * T;
         const int per = (T + BACK_OUT - 1) / BACK_OUT;
@@ -1387,7 +1423,9 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
         wgrad_args ar{};
         ar.logits = n->d_act[CNN_LAYERS];
         ar.labels = d_labels;
-        ar.next = reinterpret_cast<int *>(n->d_loss + 1);
+        ar.next = n->d_words->next;
+        ar.status = &n->d_words->status;
+        ar.lost = &n->d_words->lost;
         ar.wpos = pos_weight;
         ar.n = (int64_t)B * T;
         ar.B = B;
@@ -1427,12 +1465,40 @@ int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *n, const float *d_features,
             e = cudaGetLastError();
         }
     }
-    if (!e && loss) e = cudaMemcpyAsync(loss, n->d_loss, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream);
+    net_words words{};
+    if (!e && (loss || host_grads))
+        e = cudaMemcpyAsync(&words, n->d_words, sizeof(words), cudaMemcpyDeviceToHost, ctx->stream);
     if (!e && host_grads)
         e = cudaMemcpyAsync(host_grads, n->d_grads, (size_t)n->n_params * 4,
                             cudaMemcpyDeviceToHost, ctx->stream);
     if (!e && (loss || host_grads)) e = cudaStreamSynchronize(ctx->stream);
-    return e ? cnn_fail(ctx, e, "cnn_backward") : CETRA_OK;
+    if (e) return cnn_fail(ctx, e, "cnn_backward");
+    if (loss) *loss = words.loss;
+    return words.status ? set_error(ctx, words.status, "cnn_backward: a device wait timed out")
+                        : CETRA_OK;
+}
+
+int cetra_cnn_status(cetra_ctx *ctx, cetra_cnn *n, int *status) {
+    if (!ctx || !n || !status) return set_error(ctx, CETRA_EINVAL, "cnn_status: NULL argument");
+    device_guard dguard(ctx->device);
+    int v = 0;
+    cudaError_t e = dguard.status;
+    if (!e) e = cudaMemcpyAsync(&v, &n->d_words->status, sizeof(int), cudaMemcpyDeviceToHost,
+                                ctx->stream);
+    if (!e) e = cudaMemsetAsync(&n->d_words->status, 0, sizeof(int), ctx->stream);
+    if (!e) e = cudaStreamSynchronize(ctx->stream);
+    if (e) return cnn_fail(ctx, e, "cnn_status");
+    *status = v;
+    return CETRA_OK;
+}
+
+int cetra_selftest_cnn_waits(cetra_cnn *n, int forward_tile, int gradient_tile,
+                             int64_t wait_cycles) {
+    if (!n || wait_cycles < 0) return CETRA_EINVAL;
+    n->skip[0] = std::max(-1, forward_tile);
+    n->skip[1] = std::max(-1, gradient_tile);
+    n->wait_limit = wait_cycles ? wait_cycles : FT_WAIT_CYCLES;
+    return CETRA_OK;
 }
 
 int cetra_cnn_adam(cetra_ctx *ctx, cetra_cnn *n, float lr, float beta1, float beta2, float eps) {
@@ -1443,7 +1509,8 @@ int cetra_cnn_adam(cetra_ctx *ctx, cetra_cnn *n, float lr, float beta1, float be
     const float c1 = 1.0f - std::pow(beta1, (float)n->adam_step);
     const float c2 = 1.0f - std::pow(beta2, (float)n->adam_step);
     cnn_adam_kernel<<<(unsigned)((n->n_params + 255) / 256), 256, 0, ctx->stream>>>(
-        n->d_params, n->d_grads, n->d_m, n->d_v, n->n_params, lr, beta1, beta2, eps, c1, c2);
+        n->d_params, n->d_grads, n->d_m, n->d_v, n->n_params, lr, beta1, beta2, eps, c1, c2,
+        &n->d_words->lost);
     ctx->launches++;
     cudaError_t e = cudaGetLastError();
     if (!e) e = round_weights(ctx, n);

@@ -149,13 +149,14 @@ __device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-// Bounded wait: false if the phase did not complete within FT_WAIT_CYCLES SM clocks.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity) {
+// Bounded wait: false if the phase did not complete within `limit` SM clocks.
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
+                                          long long limit = FT_WAIT_CYCLES) {
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
         if (mbar_try(bar, parity)) return true;
-        if (clock64() - t0 > FT_WAIT_CYCLES) return false;
+        if (clock64() - t0 > limit) return false;
     }
 }
 

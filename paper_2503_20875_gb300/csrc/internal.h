@@ -235,6 +235,9 @@ size_t mono_scratch_words(const cetra_plan *plan, int max_events);
 cudaError_t launch_monotransits(cetra_ctx *ctx, const cetra_plan *plan, const float2 *ab,
                                 unsigned long long *scratch, int max_events,
                                 cetra_event *events, int *n_events);
+// The status word of a network on the device (cnn.cu): set to CETRA_ETIMEOUT, never cleared, by
+// the network's kernels.
+int *cnn_status_word(cetra_cnn *cnn);
 // Learned-proposal selection: per curve, the fold work items of its best period intervals
 // (SEL_MAX_INTERVALS intervals at most).
 constexpr int SEL_MAX_INTERVALS = 1024;

@@ -419,3 +419,65 @@ def test_forward_into_the_features(cin, T, B, shift):
     over = buf[pad + shift:pad + shift + B * T].view(B, T)
     net.forward(feats, over)
     assert torch.equal(over, own)
+
+
+def test_network_waits_that_give_up():
+    """A tile whose tensor-core work never comes (left out by the self-test; the waits are given a
+    million clocks): the tile and the block's later ones are NaN, every other probability is as
+    before, and the status word, the training step and the one-call proposal search report it.
+    Adam leaves the parameters alone, and the network works on afterwards."""
+    torch = _torch()
+    from paper_2503_20875_gb300 import CNN, CetraError
+    from paper_2503_20875_gb300 import _native as N
+    cin, T, B, tile = 4, 4096, 40, 7
+    ctx, net, p = _net(cin, T, B, seed=9)
+    f, y = _inputs(B, cin, T, seed=9)
+    d_f, d_y = torch.from_numpy(f).cuda(), torch.from_numpy(y).cuda()
+    ref = torch.empty((B, T), dtype=torch.float32, device="cuda")
+    net.forward(d_f, ref)
+    loss, g = net.backward(d_f, d_y, 5.0, grads=True)
+    assert net.status() == 0
+    # the forward pass: tiles of 230 bins, two blocks per SM
+    blocks = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    per = -(-T // 230)
+    lost = torch.zeros((B, T), dtype=torch.bool, device="cuda")
+    for k in range(tile, per * B, blocks):
+        lost[k // per, (k % per) * 230:(k % per) * 230 + 230] = True
+    assert per * B > 2 * blocks
+    net.selftest_waits(forward_tile=tile, wait_cycles=1000000)
+    out = torch.full((B, T), 2.0, dtype=torch.float32, device="cuda")
+    net.forward(d_f, out)
+    assert net.status() == N.CETRA_ETIMEOUT and net.status() == 0
+    assert bool(torch.isnan(out[lost]).all()) and torch.equal(out[~lost], ref[~lost])
+    # a training step whose forward or gradient pass gives up
+    for kw in (dict(forward_tile=tile), dict(gradient_tile=tile)):
+        net.selftest_waits(wait_cycles=1000000, **kw)
+        with pytest.raises(CetraError) as err:
+            net.backward(d_f, d_y, 5.0, grads=True)
+        assert err.value.status == N.CETRA_ETIMEOUT
+        net.adam(1e-2)
+        np.testing.assert_array_equal(net.get_params(), p)
+        # without a loss or gradients on the host only the status word tells
+        rc = N.lib.cetra_cnn_backward(ctx.handle, net.handle, d_f.data_ptr(), d_y.data_ptr(), B,
+                                      5.0, None, None)
+        assert rc == N.CETRA_OK and net.status() == N.CETRA_ETIMEOUT
+        net.adam(1e-2)
+        np.testing.assert_array_equal(net.get_params(), p)
+    # the one-call search
+    _, b, _ = _batch(3, seed=36, max_sectors=2, ratio=None)
+    other = CNN(b.ctx, b.info["n_dur"], n_bins=512, max_batch=2, seed=6)
+    other.selftest_waits(forward_tile=1, wait_cycles=1000000)
+    with pytest.raises(CetraError) as err:
+        b.search_proposed(other, n_intervals=64, top_frac=0.1)
+    assert err.value.status == N.CETRA_ETIMEOUT
+    other.selftest_waits()
+    b.search_proposed(other, n_intervals=64, top_frac=0.1)
+    # back to work
+    net.selftest_waits()
+    net.forward(d_f, out)
+    assert torch.equal(out, ref)
+    again, g2 = net.backward(d_f, d_y, 5.0, grads=True)
+    assert again == pytest.approx(loss, rel=1e-12)
+    np.testing.assert_allclose(g2, g, rtol=0, atol=1e-5 * np.abs(g).max())
+    net.adam(1e-2)
+    assert net.status() == 0 and not np.array_equal(net.get_params(), p)
