@@ -831,6 +831,9 @@ __device__ void produce_packed(fold_smem &sm, uint32_t ring0, const fold_table &
                 if (ok) mbar_expect_tx(&sm.full[rg.stage], bytes * (uint32_t)nr);
             }
             if (!__shfl_sync(0xFFFFFFFFu, (int)ok, 0)) return;
+            // the first lane's wait (the consumers' reads of the strip) comes before every lane's
+            // copies into it: the shuffle alone orders no memory
+            __syncwarp();
             fence_proxy_async();
             if (lane < nr)
                 bulk_load_s(dst + (uint32_t)lane * seg_bytes, row + a, bytes, &sm.full[rg.stage]);

@@ -188,3 +188,21 @@ def test_null_sum_is_never_a_maximum(n_points, n_dur, n_per, steps):
     g, o = gpu_search(*args, **kw), oracle_search(*args, **kw)
     assert np.isnan(g["dlogl"][-1, -1]) and np.isfinite(o["dlogl"][-1, -1])  # B = 0, A not 0
     compare_periodic(g, o, periods)
+
+
+@pytest.mark.parametrize("n_dur,precision", [(33, "fp32"), (64, "fp32"), (64, "kahan")])
+def test_packed_rows_beyond_a_warp(n_dur, precision):
+    """Strips of 33 to 64 duration rows (periods of 13 to 26 t0 steps in a launch large enough to
+    keep the durations together), so that lanes of the producer warp copy two rows each.
+    Tolerances are the parity tests' (compare_periodic)."""
+    from _parity import compare_periodic
+    from synth.lightcurves import custom
+    step = 1800.0 / 86400.0
+    periods = np.exp(np.linspace(np.log(12.6 * step), np.log(26.0 * step), 4900))
+    w = custom(seed=n_dur, n_points=700, cadence_s=1800.0,
+               durations_h=np.linspace(0.6, 6.0, n_dur), periods=periods,
+               planets=[dict(P=0.4, t0=0.1, D=0.1, depth=3e-3)])
+    args = (w.time, w.flux, w.flux_err, w.durations, w.template, periods)
+    kw = dict(cadence=w.cadence, t0_step=w.t0_step)
+    compare_periodic(gpu_search(*args, precision=precision, **kw), oracle_search(*args, **kw),
+                     periods)
