@@ -53,12 +53,13 @@ fold_kernel(const float2 *__restrict__ ab, int I, int64_t ld, int J,
         drain_copies(sm, rg);
         return;
     }
-    if (t < FT_G && k0 + t < K) {
-        const unsigned long long v = sm.best[t];
+    for (int g = t >> 5; g < FT_G && k0 + g < K; g += FT_BLOCK / 32) {  // a warp per slot
+        const unsigned long long v = slot_key(sm, g);
+        if ((t & 31) != 0) continue;
         if (!accumulate)
-            keys[k0 + t] = v;
+            keys[k0 + g] = v;
         else if (v)
-            atomicMax(&keys[k0 + t], v);
+            atomicMax(&keys[k0 + g], v);
     }
 }
 

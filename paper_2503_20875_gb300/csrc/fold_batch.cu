@@ -74,12 +74,13 @@ batch_fold_kernel(const float2 *__restrict__ ab, const batch_curve *__restrict__
             drain_copies(sm, rg);
             return;
         }
-        if (t < FT_G && k0 + t < cv.n_periods) {
-            const unsigned long long v = sm.best[t];
-            period_keys[cv.per_off + k0 + t] = v;
+        for (int g = t >> 5; g < FT_G && k0 + g < cv.n_periods; g += FT_BLOCK / 32) {
+            const unsigned long long v = slot_key(sm, g);  // a warp per slot
+            if ((t & 31) != 0) continue;
+            period_keys[cv.per_off + k0 + g] = v;
             if (v != 0ull)
                 atomicMax(&curve_keys[cidx], (v & 0xFFFFFFFF00000000ull) |
-                                                 (unsigned long long)(0xFFFFFFFFu - (uint32_t)(k0 + t)));
+                                                 (unsigned long long)(0xFFFFFFFFu - (uint32_t)(k0 + g)));
         }
     }
 }

@@ -206,3 +206,67 @@ def test_packed_rows_beyond_a_warp(n_dur, precision):
     kw = dict(cadence=w.cadence, t0_step=w.t0_step)
     compare_periodic(gpu_search(*args, precision=precision, **kw), oracle_search(*args, **kw),
                      periods)
+
+
+@pytest.mark.parametrize("n_points,n_dur,n_per,steps,gap", [
+    (900, 1, 24, (40, 440), 0),      # epoch slices
+    (2600, 3, 24, (450, 2700), 700),  # whole tiles
+    (700, 12, 4900, (13, 60), 200),  # several durations per tile
+    (20, 12, 4900, (13, 60), 0),     # the same, phases without data
+])
+def test_first_of_zeros(n_points, n_dur, n_per, steps, gap):
+    """A curve without any signal has LR 0 at every window with data: the winner is the first of
+    them in (duration, phase) order, also where the first phases hold none, with a mask, and for
+    a curve of a batch."""
+    from paper_2503_20875_gb300 import Batch, Context
+    from synth.lightcurves import custom
+    c = 120.0 / 86400.0
+    periods = np.exp(np.linspace(np.log(steps[0] * c), np.log(steps[1] * c), n_per))
+    w = custom(seed=n_points, n_points=n_points, cadence_s=120.0, gaps=[(3 * c, (3 + gap) * c)],
+               durations_h=np.linspace(0.1, 0.4, n_dur), periods=periods)
+    w.flux[:] = 1.0
+    args = (w.time, w.flux, w.flux_err, w.durations, w.template, periods)
+    kw = dict(cadence=c, t0_step=c)
+    mask = (np.random.default_rng(n_dur).uniform(size=(n_per, n_dur)) < 0.5).astype(np.uint8)
+    for m in (None, mask):
+        g, o = gpu_search(*args, mask=m, **kw), oracle_search(*args, mask=m, **kw)
+        for key in ("dlogl", "i", "j"):
+            np.testing.assert_array_equal(g["periodic"][key], o["periodic"][key])
+    b = Batch(Context(0), [(w.time, w.flux, w.flux_err)] * 2, w.durations, w.template,
+              periods[0], periods[-1], periods[1] / periods[0], cadence=c, t0_step=c)
+    best = b.run()
+    o = oracle_search(*args, **kw)["periodic"]
+    first = int(np.flatnonzero(~np.isnan(o["dlogl"]))[0])
+    for x in range(2):
+        assert (best["k"][x], best["i"][x], best["j"][x], best["dlogl"][x]) == (
+            first, o["i"][first], o["j"][first], 0.0)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "kahan"])
+def test_a_flat_curve_is_no_slower(precision):
+    """Windows without any signal are no candidates for a period's maximum: the search of a flat
+    curve may not take longer than a noisy one's (1.2 x, for the timer's sake; least of ten)."""
+    import torch
+    import synth
+    from paper_2503_20875_gb300 import Context, DeviceSearch, Plan
+    from synth.lightcurves import custom
+    w = custom(seed=4, n_points=60000, cadence_s=20.0, durations_h=np.linspace(0.5, 12.0, 20))
+    periods = synth.log_grid(0.5, 6.5, 6000)
+    ctx = Context(0)
+    plan = Plan(ctx, w.time, w.flux, w.flux_err, w.durations, w.template, cadence=w.cadence,
+                t0_step=w.t0_step, precision=precision)
+    ds = DeviceSearch(ctx, plan, periods)
+    t, f, e = (torch.from_numpy(np.ascontiguousarray(x)).cuda()
+               for x in (w.time, w.flux, w.flux_err))
+    took = {}
+    for name, flux in (("noisy", f), ("flat", torch.ones_like(f))):
+        ms = []
+        for _ in range(13):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ds.run(t, flux, e)
+            b.record()
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(b))
+        took[name] = min(ms[3:])
+    assert took["flat"] <= 1.2 * took["noisy"], took
