@@ -421,6 +421,41 @@ def test_forward_into_the_features(cin, T, B, shift):
     assert torch.equal(over, own)
 
 
+def test_network_sums_are_not_one_sided():
+    """The tensor cores' accumulators truncate, which must not shift what averages over bins. One
+    network's logits and gradients are off by some 5e-8 of their size to either side even with
+    FP32 sums (the bins share the weights and with them the roundings), so the shift is averaged
+    over 12 networks: below half a unit in the last place (2^-24) for the logits, and a unit
+    (2^-23) for the scale of the last layer's gradient, whose activations all carry the shift of
+    three layers."""
+    torch = _torch()
+    from paper_2503_20875_gb300 import CNN, Context
+    B, T = 4, 1024
+    shifts, scales = [], []
+    for cin in (8, 16, 32):
+        for seed in range(cin, cin + 4):
+            net = CNN(Context(0), cin, n_bins=T, max_batch=B, seed=seed)
+            p = net.get_params()  # He-normal weights
+            p += np.random.default_rng(seed).normal(0.0, 0.02, p.size).astype(np.float32)
+            net.set_params(p)
+            f, y = _inputs(B, cin, T, seed=60 + seed)
+            d_f = torch.from_numpy(f).cuda()
+            prob = torch.empty((B, T), dtype=torch.float32, device="cuda")
+            net.forward(d_f, prob)
+            acts, _, _ = ocnn.forward(p, f)
+            ref, got = acts[-1][:, 0, :], prob.cpu().numpy().astype(np.float64)
+            ok = np.abs(ref) < 3.0  # a probability near 1 does not hold its logit
+            z = np.log(got[ok] / (1.0 - got[ok]))
+            shifts.append(np.sum(np.sign(ref[ok]) * (z - ref[ok])) / np.sum(np.abs(ref[ok])))
+            _, g = net.backward(d_f, torch.from_numpy(y).cuda(), 20.0, grads=True)
+            _, ref_g = ocnn.loss_and_grads(p, f, y, 20.0)
+            last = _layer_slices(cin)[-1]
+            a, b = g[last].astype(np.float64), ref_g[last]
+            scales.append(a @ b / (b @ b) - 1.0)
+    assert abs(np.mean(shifts)) <= 2.0 ** -24, shifts
+    assert abs(np.mean(scales)) <= 2.0 ** -23, scales
+
+
 def test_network_waits_that_give_up():
     """A tile whose tensor-core work never comes (left out by the self-test; the waits are given a
     million clocks): the tile and the block's later ones are NaN, every other probability is as
