@@ -516,3 +516,50 @@ def test_network_waits_that_give_up():
     np.testing.assert_allclose(g2, g, rtol=0, atol=1e-5 * np.abs(g).max())
     net.adam(1e-2)
     assert net.status() == 0 and not np.array_equal(net.get_params(), p)
+
+
+def _check_gradients(p, f, y, w_pos, loss, g):
+    """Against the FP64 reference on f, y, with the tolerances of test_gradients_match_oracle."""
+    ref_loss, ref_g = ocnn.loss_and_grads(p, f, y, w_pos)
+    assert loss == pytest.approx(ref_loss, rel=1e-5)
+    for sl in _layer_slices(f.shape[1]):
+        np.testing.assert_allclose(g[sl], ref_g[sl], rtol=0, atol=2e-3 * np.abs(ref_g[sl]).max())
+
+
+@pytest.mark.parametrize("cin,T,B", [(17, 768, 2), (24, 256, 1), (32, 1024, 3)])
+def test_gradients_of_wide_inputs(cin, T, B):
+    """17 to 32 input channels: the first layer's weight gradients hold 32 channels and half as
+    many bins per tile; every last tile is ragged."""
+    torch = _torch()
+    _, net, p = _net(cin, T, B, seed=50 + cin)
+    f, y = _inputs(B, cin, T, seed=cin)
+    loss, g = net.backward(torch.from_numpy(f).cuda(), torch.from_numpy(y).cuda(), 8.0,
+                           grads=True)
+    _check_gradients(p, f, y, 8.0, loss, g)
+
+
+@pytest.mark.parametrize("cin", [16, 32])
+def test_more_tiles_than_blocks(cin):
+    """48 curves of 4,096 bins are 864 tiles, three for each of the blocks that two per SM make:
+    the next tile's input read ahead, the barriers' parity carried on, and the weight gradients'
+    tiles handed out. Two curves in turn: every copy of a curve has the same bits, the two match
+    the reference, and the batch's mean loss and gradients are those of the two. He-normal weights
+    (logits of order 1, as the tolerance of test_forward_matches_oracle has them)."""
+    torch = _torch()
+    from paper_2503_20875_gb300 import CNN, Context
+    T, B = 4096, 48
+    net = CNN(Context(0), cin, n_bins=T, max_batch=B, seed=70 + cin)
+    p = net.get_params()
+    p += np.random.default_rng(cin).normal(0.0, 0.02, p.size).astype(np.float32)  # biases too
+    net.set_params(p)
+    f, y = _inputs(2, cin, T, seed=cin)
+    d_f = torch.from_numpy(f).cuda().repeat(B // 2, 1, 1)
+    d_y = torch.from_numpy(y).cuda().repeat(B // 2, 1)
+    assert B * -(-T // 230) > 2 * 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    out = torch.empty((B, T), dtype=torch.float32, device="cuda")
+    net.forward(d_f, out)
+    got = out.cpu().numpy()
+    np.testing.assert_allclose(got[:2], ocnn.probabilities(p, f), rtol=0, atol=2e-5)
+    np.testing.assert_array_equal(got, np.tile(got[:2], (B // 2, 1)))
+    loss, g = net.backward(d_f, d_y, 8.0, grads=True)
+    _check_gradients(p, f, y, 8.0, loss, g)
