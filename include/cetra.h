@@ -445,9 +445,9 @@ int cetra_cnn_forward(cetra_ctx *ctx, cetra_cnn *cnn, const float *d_features, i
 /* Forward + backward of the weighted binary cross-entropy with logits against d_labels
  * (device FP32 [B][n_bins], 0 or 1), mean over bins, positive weight pos_weight. Leaves the
  * gradient on the device for cetra_cnn_adam; *loss and host_grads (flat, like the
- * parameters) are filled when not NULL (that synchronises). Weight gradients are summed with
- * atomics, so their last bits may differ from run to run. Where a bounded device wait gave up,
- * loss and gradient are NaN and cetra_cnn_status says so.
+ * parameters) are filled when not NULL (that synchronises). Tiles of bins are handed to blocks as
+ * these come free and the loss is summed with FP64 atomics, so last bits may differ from run to
+ * run. Where a bounded device wait gave up, loss and gradient are NaN and cetra_cnn_status says so.
  * Errors as cetra_cnn_forward, and CETRA_ETIMEOUT when it synchronised and a wait gave up. */
 int cetra_cnn_backward(cetra_ctx *ctx, cetra_cnn *cnn, const float *d_features,
                        const float *d_labels, int B, float pos_weight, double *loss,

@@ -47,16 +47,14 @@ constexpr size_t kCombSmemMax = 98 * 1024;  // maps up to 24,576 bins (+ 512 cel
 //
 // Measured (256 curves, 16 durations, 4,096 bins): 2,347 us as log1p, four FP32 conv kernels and
 // a sigmoid with every activation in memory, 260 us as this kernel (three parts' products alone:
-// 76 us at the measured BF16 rate). Bound: the instructions' reads of the activations and the
-// epilogues (splitting the next layer's input), in turn between the two blocks of an SM.
+// 76 us at the measured BF16 rate). Bound: the instructions' reads of the activation operand from
+// shared memory (4 KB each, 150 per tile at 16 durations) and the epilogues (splitting the next
+// layer's input), in turn: two blocks per SM, so that one's epilogue runs under the other's
+// instructions.
 //
 // Halo: layer l's row r is bin t0 - 16 + 4 l + r. A tile computes NET_ROWS = 254 rows of the
 // first three layers in place (rows past the last valid one are never used): 254, 246, 238
 // valid rows, then NET_OUT = 230 logits. Rows outside [0, T) are zero (zero padding).
-//
-// Bound: reading the activation operand from shared memory (4 KB per instruction): 150
-// instructions per tile at 16 durations. Two blocks per SM, so that one's epilogue runs under the
-// other's matrix instructions.
 constexpr int NET_BLOCK = 127;             // rows a block of 128 completes (see net_layer_mma)
 constexpr int NET_ROWS = 2 * NET_BLOCK;    // rows computed per layer
 constexpr int NET_XROWS = 264;             // rows held: 8 more for the last tap, whole groups of 8

@@ -965,7 +965,7 @@ template <int GS, int R, int W, bool KAHAN>
 __device__ __forceinline__ bool packed_tile_rows(int rows, fold_smem &sm, uint32_t ring0,
                                                  const fold_table &tb, int g0, int Tp, int H,
                                                  int seg, int t0, int nr, int nE, ring &rg) {
-    if constexpr (R > 1 && !KAHAN) {  // (the compensated form's tiles are half as wide)
+    if constexpr (R > 1 && !KAHAN) {  // (compensated: 336.2 -> 337.5 ms for 24 curves, not worth it)
         if (rows < R)
             return packed_tile_rows<GS, R - 1, W, KAHAN>(rows, sm, ring0, tb, g0, Tp, H, seg, t0,
                                                          nr, nE, rg);
@@ -1295,6 +1295,8 @@ __device__ __forceinline__ void fold_group(fold_smem &sm, unsigned char *raw, un
     }
 }
 
+// Dynamic shared memory of the kernels: the strip ring, then the epoch table (fold_smem_bytes).
+//
 // Block start: barriers (the full ones expect the producer's one arrival, the empty ones one
 // arrival per consumer thread).
 __device__ __forceinline__ void fold_init_barriers(fold_smem &sm) {
@@ -1315,7 +1317,5 @@ __device__ void drain_copies(fold_smem &sm, const ring &rg) {
     if (threadIdx.x != FT_THREADS) return;  // the producer's issuing lane holds the ring state
     for (int s = 0; s < FT_NSTAGE; ++s) mbar_wait(&sm.full[s], ((rg.par >> s) & 1u) ^ 1u);
 }
-
-// Dynamic shared memory: the strip ring, then the epoch table.
 
 }  // namespace
