@@ -292,9 +292,17 @@ __device__ __forceinline__ void issue_copy(fold_smem &sm, uint32_t ring0, const 
 // candidates (with -1 there too, the exact values of every tile made the fold of a flat 20-s curve
 // 1.6 x as long as a noisy one's: 10,000 of its periods 9.9 ms, now 5.9 ms). Which of equal zeros
 // is the first is worked out for the slots that end with one (zero_winner).
-__device__ __forceinline__ float candidate_factor(uint32_t lr_bits) {
+//
+// The test compares x^2 with h y, which underflow where the weights are tiny (flux errors of 1e8
+// and above). It decides rightly while b y 2^-14 is above the smallest float, 2^-149, so h leaves
+// -1 only for maxima far above that, y being the B of the maximum's window or a neighbour's:
+// b y >= 2^-100 (windows of 2^-35 times that B still pass), or b = 0 and y >= 1 (what underflows
+// then has LR zero). Otherwise the exact values decide. (As one product; with two comparisons the
+// compensated fold was 1 % slower.)
+__device__ __forceinline__ float candidate_factor(uint32_t lr_bits, float y) {
     const float b = 2.0f * __uint_as_float(lr_bits);
-    return b < INFINITY ? b * kCandidate : -1.0f;
+    const bool sure = (b > 0.0f ? b * 0x1p100f : 1.0f) * y >= 1.0f;
+    return sure && b < INFINITY ? b * kCandidate : -1.0f;
 }
 template <int GS>
 __device__ __forceinline__ void load_factors(const fold_smem &sm, int g0, float (&h)[GS]) {
@@ -318,8 +326,9 @@ __device__ __forceinline__ float load_factor(const fold_smem &sm, int g) {
 
 // Offer slot g the best window of each lane of a warp (called by whole warps): 2 LR = lr2 at
 // flat index at; a lane without one passes lr2 < 0. The larger LR stays, on equal LR the smaller
-// flat index (make_key).
-__device__ __forceinline__ void offer_best(fold_smem &sm, int g, float lr2, uint32_t at) {
+// flat index (make_key). top_y(): the largest B of the lane's windows (a slot's few updates only).
+template <class F>
+__device__ __forceinline__ void offer_best(fold_smem &sm, int g, float lr2, uint32_t at, F top_y) {
     const uint32_t v = lr2 >= 0.0f ? __float_as_uint(0.5f * lr2) + 1u : 0u;  // 0: none
     const uint32_t top = __reduce_max_sync(0xFFFFFFFFu, v);
     if (top == 0u) return;
@@ -328,9 +337,22 @@ __device__ __forceinline__ void offer_best(fold_smem &sm, int g, float lr2, uint
             ((unsigned long long)(top - 1u) << 32) | (unsigned long long)(0xFFFFFFFFu - at);
         if (key > *(volatile unsigned long long *)&sm.best[g]) {
             atomicMax(&sm.best[g], key);
-            atomicMax(&sm.factor[g], __float_as_int(candidate_factor(top - 1u)));
+            atomicMax(&sm.factor[g], __float_as_int(candidate_factor(top - 1u, top_y())));
         }
     }
+}
+
+// The largest B of a lane's windows of one period.
+template <int R>
+__device__ __forceinline__ float largest_b(const uint64_t (&acc)[R]) {
+    float top = 0.0f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float x, y;
+        split_pair(acc[r], x, y);
+        top = fmaxf(top, y);
+    }
+    return top;
 }
 
 // The better of a lane's best window (lr2, at) and the window sum (x, y) at index here, which
@@ -592,7 +614,7 @@ __device__ __forceinline__ bool consume_tile(fold_smem &sm, const fold_table &tb
                 if (i0 + c + r * FT_THREADS < nph)
                     take_max(x, y, at0 + (uint32_t)(r * FT_THREADS), lr2, at);
             }
-            offer_best(sm, g0 + gg, lr2, at);
+            offer_best(sm, g0 + gg, lr2, at, [&] { return largest_b(acc[gg]); });
         }
     }
     return true;
@@ -759,7 +781,7 @@ __device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part,
             }
             block_sync();
             const int nph = sm.nph[g0 + gg];
-            float lr2 = -1.0f;
+            float lr2 = -1.0f, top = 0.0f;
             uint32_t at = 0u;
             for (int phi = c; phi < min(Tp, nph); phi += FT_THREADS) {
                 uint64_t v = part[phi];
@@ -767,9 +789,10 @@ __device__ void consume_sliced(fold_smem &sm, uint32_t ring0, uint64_t *part,
                 float x, y;
                 split_pair(v, x, y);
                 take_max(x, y, (uint32_t)j * (uint32_t)I + (uint32_t)phi, lr2, at);
+                top = fmaxf(top, y);
             }
             if (__any_sync(0xFFFFFFFFu, lr2 > load_factor(sm, g0 + gg)))
-                offer_best(sm, g0 + gg, lr2, at);
+                offer_best(sm, g0 + gg, lr2, at, [&] { return top; });
             block_sync();
         }
     }
@@ -954,7 +977,7 @@ __device__ __forceinline__ bool packed_tile(fold_smem &sm, uint32_t ring0, const
             split_pair(v, x, y);
             take_max(x, y, (uint32_t)sm.pack_j[t0 + row] * I + (uint32_t)ph, lr2, at);
         }
-        offer_best(sm, g0 + gg, lr2, at);
+        offer_best(sm, g0 + gg, lr2, at, [&] { return largest_b(acc[gg]); });
     }
     return true;
 }
@@ -1079,7 +1102,9 @@ __device__ __forceinline__ void fold_slot_meta(fold_smem &sm, int t, bool presen
     sm.nph[t] = nph;
     sm.E[t] = E;
     sm.best[t] = 0ull;
-    sm.factor[t] = __float_as_int(floor_lr ? candidate_factor(floor_lr) : -1.0f);
+    // (of the floor's window no B is known: at 2^-9 and above any will do)
+    sm.factor[t] = __float_as_int(
+        __uint_as_float(floor_lr) >= 0x1p-9f ? candidate_factor(floor_lr, 1.0f) : -1.0f);
 }
 
 // Build the epoch table of sub-group [g0, g0 + GS) (all threads), offsets W bytes wide. Sets

@@ -270,3 +270,40 @@ def test_a_flat_curve_is_no_slower(precision):
             ms.append(a.elapsed_time(b))
         took[name] = min(ms[3:])
     assert took["flat"] <= 1.2 * took["noisy"], took
+
+
+@pytest.mark.parametrize("n_points,n_dur,n_per,steps", [
+    (900, 1, 24, (40, 440)),      # epoch slices
+    (2600, 3, 24, (450, 2700)),   # whole tiles
+    (700, 12, 4900, (13, 60)),    # several durations per tile
+])
+@pytest.mark.parametrize("flat", [False, True])
+@pytest.mark.parametrize("power", [40, 48])
+def test_winners_do_not_depend_on_the_errors_unit(n_points, n_dur, n_per, steps, flat, power):
+    """Flux errors 2^40 and 2^48 times as large scale every window's (A, B) by a power of two, and
+    LR with it: the same winners, their LR scaled exactly, although A^2 falls below the smallest
+    float. Flat: all windows but those that hold one point have LR 0."""
+    from paper_2503_20875_gb300 import Batch, Context
+    from synth.lightcurves import custom
+    c = 120.0 / 86400.0
+    periods = np.exp(np.linspace(np.log(steps[0] * c), np.log(steps[1] * c), n_per))
+    w = custom(seed=power + n_points, n_points=n_points, cadence_s=120.0, sigma_spread=0.3,
+               durations_h=np.linspace(0.1, 0.4, n_dur), periods=periods)
+    if flat:
+        w.flux[:] = 1.0
+        w.flux[2 * n_points // 3] = np.float32(0.999)
+    scale = np.float32(2.0 ** power)
+    out = []
+    for err in (w.flux_err, w.flux_err * scale):
+        g = gpu_search(w.time, w.flux, err, w.durations, w.template, periods, cadence=c,
+                       t0_step=c)["periodic"]
+        b = Batch(Context(0), [(w.time, w.flux, err)], w.durations, w.template, periods[0],
+                  periods[-1], periods[1] / periods[0], cadence=c, t0_step=c).run()
+        out.append((g, b))
+    (g0, b0), (g1, b1) = out
+    for key in ("i", "j"):
+        np.testing.assert_array_equal(g1[key], g0[key])
+        np.testing.assert_array_equal(b1[key], b0[key])
+    np.testing.assert_array_equal(g1["dlogl"] * 4.0 ** power, g0["dlogl"])
+    np.testing.assert_array_equal(b1["dlogl"] * 4.0 ** power, b0["dlogl"])
+    np.testing.assert_array_equal(b1["k"], b0["k"])
